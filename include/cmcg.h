@@ -130,18 +130,18 @@ typedef struct cmcg_mesh {
  *   device:           CUDA device ordinal.
  *   stage_variant:    0 = time the stage-kernel forms on this mesh at
  *                     creation and keep the fastest; k > 0 forces form k - 1.
- *                     FP32: 0, 1, 2 = two threads per tetrahedron (E / H)
- *                     with at least 1, 3, 4 resident 128-thread blocks per
- *                     SM; 3, 4, 5 = four threads per tetrahedron (E / H x
- *                     node half) with at least 4, 5, 6; 6 = the volume and
- *                     lift contractions on the tensor cores (tcgen05, three
- *                     TF32 products per FP32 product, FP32 accumulation),
- *                     two threads per tetrahedron.  FP64: 0 = two threads
- *                     per tetrahedron; 1, 2 = four threads with at least
- *                     2, 3.  Other k: CMCG_ERR_INVALID_ARG.  Results do not
+ *                     FP32: 0, 1, 2 = two threads per tetrahedron (E / H),
+ *                     one warp per 16 tetrahedra, with at least 3, 4, 6
+ *                     resident 128-thread blocks per SM; 3, 4 = two warps
+ *                     per 16 tetrahedra with at least 3, 4; 5 = four warps;
+ *                     6 = the volume and lift contractions on the tensor
+ *                     cores (tcgen05, three TF32 products per FP32 product,
+ *                     FP32 accumulation).  Forms 0 to 5 give the same bits;
+ *                     0 times those at orders 1 and 2 and takes form 6 at
+ *                     order 3.  FP64: 0, 1, 2 = one, two, four warps per 16
+ *                     tetrahedra.  Other k: CMCG_ERR_INVALID_ARG.  Results do not
  *                     depend on it beyond rounding.
- *   stage_overlap:    0 = decide by timing when the form is timed (on when
- *                     the form is forced); 1 = on; 2 = off.  On: each stage
+ *   stage_overlap:    0 or 1 = on; 2 = off.  On: each stage
  *                     is launched with programmatic stream serialisation, so
  *                     its blocks start and load the mesh data while the
  *                     previous stage finishes.  Results are identical.
@@ -274,9 +274,9 @@ int cmcg_set_stream(cmcg_handle* h, void* stream);
 
 /* Stage-kernel form in use (0-based, as stage_variant - 1) and, when it was
  * chosen by timing at creation, the measured microseconds per stage of each
- * form (10 entries: [0..6] indexed by form, see stage_variant; [7] the chosen
- * form with stage_overlap on; [8], [9] unused; -1 where not timed or rejected by
- * the device).  Any pointer may be NULL. */
+ * form (10 entries: [0..6] indexed by form, see stage_variant, launched as the
+ * sweeps launch them; [7] the chosen form; [8], [9] unused; -1 where not timed
+ * or rejected by the device).  Any pointer may be NULL. */
 int cmcg_get_tuning(const cmcg_handle* h, int* variant, double* us_per_stage);
 
 /* Sizes of the handle: nt, Np, M (steps per period), dt, number of doubles of
@@ -415,7 +415,8 @@ int cmcg_slot_state(const cmcg_handle* h, int slot);
  * handle whose problem in that slot has the same mesh size, order, precision,
  * M, dt and omega (else CMCG_ERR_INVALID_ARG); the request then continues as
  * if it had never stopped (the same bits).  The state is in the handle's
- * internal layout and precision, for the same library build. */
+ * internal layout and precision, for the same library build; states of the
+ * first layout (nodal values, magic CMCGSLT1) are converted. */
 int64_t cmcg_slot_state_bytes(const cmcg_handle* h, int slot);
 int cmcg_slot_save(cmcg_handle* h, int slot, void* buf, int64_t len);
 int cmcg_slot_restore(cmcg_handle* h, int slot, const void* buf, int64_t len);

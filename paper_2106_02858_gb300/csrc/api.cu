@@ -42,7 +42,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
-#include "common.h"
+#include "bernstein.h"
 
 using namespace cmcg;
 
@@ -59,14 +59,22 @@ struct Range {
 
 namespace {
 
-// An impedance face of a problem: what its boundary data need on the host.
-struct ImpFace {
-  int64_t it = 0;        // internal tetrahedron (handle-wide index)
-  int32_t ext = 0;       // external tetrahedron within its problem
-  int f = 0;             // face
-  double n[3] = {0, 0, 0};
-  double aE = 0, bH = 0;  // flux coefficients of the E rows (tangential jump) and H rows (n x jump)
-};
+// Nodal values -> Bernstein coefficients of consecutive components of Np values each.
+template <typename T>
+void to_bern_rows(int q, std::vector<T>& x) {
+  const int np = np_of(q);
+  std::vector<BasisTab> rows;
+  for (int n = 0; n < np; ++n) rows.push_back(to_bern_row(q, n));
+  std::vector<double> u(size_t(np), 0.0);
+  for (size_t o = 0; o + np <= x.size(); o += np) {
+    for (int n = 0; n < np; ++n) u[n] = double(x[o + n]);
+    for (int n = 0; n < np; ++n) {
+      double v = 0;
+      for (int k = 0; k < rows[n].n; ++k) v += rows[n].w[k] * u[rows[n].col[k]];
+      x[o + n] = T(v);
+    }
+  }
+}
 
 struct Prob {
   int64_t nt = 0;                     // external tetrahedra
@@ -81,6 +89,7 @@ struct Prob {
   bool has_sigma = false;                     // conductivity set (cmcg_set_conductivity)
   std::vector<int32_t> ext_of_int;            // internal (problem-local) -> external tetrahedron (-1 padding)
   std::vector<int32_t> int_of_ext;            // external -> internal (problem-local)
+  std::vector<int32_t> half_at;               // half tile in the order of the shape classes -> internal half tile
 };
 
 }  // namespace
@@ -90,11 +99,11 @@ struct cmcg_handle {
   cudaStream_t stream = nullptr;
   int q = 1, np = 4, prec = CMCG_FP64, s = 2, nprob = 1;
   std::vector<Prob> P;
-  int64_t nti = 0, ntiles = 0, nvec = 0, njvec = 0, nt_total = 0;
+  int64_t nti = 0, ntiles = 0, nvec = 0, nt_total = 0;
   size_t rsize = 8;
   int maxM = 0;
   // device geometry
-  void *gvol = nullptr, *gface = nullptr;
+  void* geo = nullptr;
   int32_t* nbr = nullptr;
   double* wdot = nullptr;
   int32_t* e_of_i = nullptr;  // internal tet -> external index within its problem (-1 = padding)
@@ -102,7 +111,7 @@ struct cmcg_handle {
   double* inv_eps = nullptr;  // external order, problems concatenated
   // vectors
   void *Uw = nullptr, *vA = nullptr, *vB = nullptr, *Fre = nullptr, *Fim = nullptr;
-  void *Jre = nullptr, *Jim = nullptr;
+  void* J = nullptr;                    // source: J_re at the electric, J_im at the magnetic places
   void *Bre = nullptr, *Bim = nullptr;  // lifted impedance-face data, all 6 rows (allocated on first use)
   void *U0 = nullptr, *Rv = nullptr, *D = nullptr, *A = nullptr, *WT = nullptr;
   // CG
@@ -114,7 +123,7 @@ struct cmcg_handle {
   int32_t* used = nullptr;          // problems taking part in the current solve
   int32_t* used_host = nullptr;     // pinned
   int64_t* bt_tet0 = nullptr;
-  int32_t *bt_ntet = nullptr, *bt_prob = nullptr, *bt_pb0 = nullptr;
+  int32_t *bt_half = nullptr, *bt_ntet = nullptr, *bt_prob = nullptr, *bt_pb0 = nullptr;
   BlockTable bt{};
   // per-launch coefficient tables
   void *tab_free = nullptr, *tab_src = nullptr, *tab_srcf = nullptr, *tab_one = nullptr;
@@ -135,10 +144,10 @@ struct cmcg_handle {
   int32_t *g_in = nullptr, *g_out = nullptr;          // internal -> global tetrahedron (g_out: owned only)
   double* inv_eps_g = nullptr;                        // 1 / eps by global tetrahedron
   // Several harmonics in one solve (cmcg_solve_multifreq): while mf_nharm > 0 the source sweeps
-  // read mf_nharm sources from Jm_re / Jm_im (njvec values apart) with the per-launch harmonic
+  // read mf_nharm sources from Jm (nvec values apart) with the per-launch harmonic
   // coefficients mf_hcs, and filtered sweeps use the filter table mf_tab of the harmonic being read.
   int mf_nharm = 0, mf_cap = 0;
-  void *Jm_re = nullptr, *Jm_im = nullptr, *mf_hcs = nullptr, *mf_tab = nullptr;
+  void *Jm = nullptr, *mf_hcs = nullptr, *mf_tab = nullptr;
   double* mf_src = nullptr;  // host sources of cmcg_solve_multifreq, on the device
   size_t mf_src_len = 0;
   // Slots (continuous batching, cmcg_slot_*): phase of every problem and the per-phase masks.
@@ -335,8 +344,7 @@ const StageCoef<R>* tab(void* t, int l, int nprob) {
 
 template <typename R>
 void stage(cmcg_handle* h, StageArgs<R>& a, cudaStream_t st) {
-  a.gvol = (const R*)h->gvol;
-  a.gface = (const R*)h->gface;
+  a.geo = (const R*)h->geo;
   a.nbr = h->nbr;
   a.nti = h->nti;
   a.err = h->err;
@@ -482,11 +490,10 @@ void sweep_source(cmcg_handle* h, bool with_source, bool filter, const int32_t* 
     a.base = Uw;
     a.out = r == s - 1 ? Uw : (r % 2 == 0 ? vA : vB);
     if (with_source) {
-      a.jre = (const R*)(K > 0 ? h->Jm_re : h->Jre);
-      a.jim = (const R*)(K > 0 ? h->Jm_im : h->Jim);
+      a.j = (const R*)(K > 0 ? h->Jm : h->J);
       if (K > 0) {
         a.nharm = K;
-        a.jstride = h->njvec;
+        a.jstride = h->nvec;
         a.hcs = (const R*)h->mf_hcs + size_t(l) * 2 * K;
       }
       if (h->has_bdata) {
@@ -513,11 +520,14 @@ void sweep_source(cmcg_handle* h, bool with_source, bool filter, const int32_t* 
   prof_end(h, pe);
 }
 
-// Times the stage-kernel forms on this batch with a nested source-free stage
-// on zero fields (3 warm-up + 12 timed launches each) and keeps the fastest;
-// tune_us[f] is the time of form f (-1: not timed or rejected by the device).
+// Times the stage-kernel forms [first, first + nforms) on this batch with a nested source-free stage
+// on zero fields (3 warm-up + 12 timed launches each), launched as the sweeps launch them (overlapped
+// unless the caller forbids it: launches that wait for each other end on a 2 us raster that hides
+// what tells small forms apart), and keeps the fastest; tune_us[f] is the time of form f (-1: not
+// timed or rejected by the device), tune_us[7] that of the chosen form.  The forms of one range give
+// the same bits.
 template <typename R>
-int autotune(cmcg_handle* h, int nforms, int overlap) {
+int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
   for (double& x : h->tune_us) x = -1;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
@@ -554,8 +564,9 @@ int autotune(cmcg_handle* h, int nforms, int overlap) {
   };
   double best = 1e300;
   int bestf = 0;
-  h->pdl = false;
-  for (int f = 0; f < nforms; ++f) {
+  h->pdl = overlap != 2;
+  bestf = first;
+  for (int f = first; f < first + nforms; ++f) {
     h->form = f;
     double us;
     int rc = time_one(&us);
@@ -567,16 +578,7 @@ int autotune(cmcg_handle* h, int nforms, int overlap) {
     }
   }
   h->form = bestf;
-  if (overlap == 0) {  // the chosen form with overlapped stage launches
-    h->pdl = true;
-    double us;
-    int rc = time_one(&us);
-    if (rc) return rc;
-    h->tune_us[7] = us;
-    h->pdl = us >= 0 && us < best;
-  } else {
-    h->pdl = overlap == 1;
-  }
+  h->tune_us[7] = h->tune_us[bestf];
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   h->launches = launches0;
@@ -588,22 +590,40 @@ int autotune(cmcg_handle* h, int nforms, int overlap) {
 // (For a sharded handle the external arrays are the global mesh's: every part reads its owned
 // and ghost tetrahedra and writes its owned ones.)
 template <typename R>
-void to_int(cmcg_handle* h, int p, const double* ext, int ncomp_ext, void* in, int ncomp_in, int cnt,
-            const double* per_tet) {
+void to_int(cmcg_handle* h, int p, const double* x0, const double* x1, int64_t stride, void* in, const double* per_tet) {
   const Prob& P = h->P[p];
-  R* base = (R*)in + P.tile0 * int64_t(ncomp_in) * h->np * TILE;
+  R* base = (R*)in + P.tet0 * 6 * h->np;
   const int32_t* map = h->coupled ? h->g_in + P.tet0 : h->e_of_i + P.tet0;
   const double* pt = per_tet ? (h->coupled ? h->inv_eps_g : per_tet + P.ext0) : nullptr;
-  launch_to_internal<R>(ext, ncomp_ext, 0, base, ncomp_in, 0, cnt, map, P.nti, h->np, 1.0, pt, h->stream);
+  launch_to_internal<R>(h->q, x0, x1, stride, base, map, P.nti, pt, h->stream);
   h->launches++;
 }
 template <typename R>
-void to_ext(cmcg_handle* h, int p, const void* in, int ncomp_in, int c_in0, double* ext, int ncomp_ext, int cnt) {
+void to_ext(cmcg_handle* h, int p, const void* in, double* x0, double* x1, int64_t stride) {
   const Prob& P = h->P[p];
-  const R* base = (const R*)in + P.tile0 * int64_t(ncomp_in) * h->np * TILE;
+  const R* base = (const R*)in + P.tet0 * 6 * h->np;
   const int32_t* map = h->coupled ? h->g_out + P.tet0 : h->e_of_i + P.tet0;
-  launch_to_external<R>(base, ncomp_in, c_in0, ext, ncomp_ext, 0, cnt, map, P.nti, h->np, h->stream);
+  launch_to_external<R>(h->q, base, x0, x1, stride, map, P.nti, h->stream);
   h->launches++;
+}
+// A six-component array [tet][6][Np], and the source arrays [tet][3][Np] (im null: real).
+template <typename R>
+void field_to_int(cmcg_handle* h, int p, const double* u, void* in) {
+  to_int<R>(h, p, u, u + 3 * h->np, int64_t(6) * h->np, in, nullptr);
+}
+template <typename R>
+void field_to_ext(cmcg_handle* h, int p, const void* in, double* u) {
+  to_ext<R>(h, p, in, u, u + 3 * h->np, int64_t(6) * h->np);
+}
+template <typename R>
+void source_to_int(cmcg_handle* h, int p, const double* re, const double* im, void* in) {
+  to_int<R>(h, p, re, im, int64_t(3) * h->np, in, h->inv_eps);
+}
+// The filtered field's real and imaginary parts, E and H apart ([tet][3][Np] each).
+template <typename R>
+void filtered_to_ext(cmcg_handle* h, int p, double* e_re, double* e_im, double* h_re, double* h_im) {
+  to_ext<R>(h, p, h->Fre, e_re, h_re, int64_t(3) * h->np);
+  to_ext<R>(h, p, h->Fim, e_im, h_im, int64_t(3) * h->np);
 }
 // Number of problems a single-problem entry point converts: all parts of a sharded handle.
 int nconv(const cmcg_handle* h) { return h->coupled ? h->nprob : 1; }
@@ -616,19 +636,9 @@ void lincomb(cmcg_handle* h, void* o1, void* o2, void* o3, double a, const void*
 }
 
 template <typename R>
-int set_source(cmcg_handle* h, const double* const* j_re, const double* const* j_im, int nused = -1) {
-  for (int p = 0; p < (nused < 0 ? h->nprob : nused); ++p) {
-    to_int<R>(h, p, j_re[p], 3, h->Jre, 3, 3, h->inv_eps);
-    const double* ji = j_im ? j_im[p] : nullptr;
-    if (ji) {
-      to_int<R>(h, p, ji, 3, h->Jim, 3, 3, h->inv_eps);
-    } else {
-      const Prob& P = h->P[p];
-      CK(cudaMemsetAsync((char*)h->Jim + P.tile0 * 3 * h->np * TILE * h->rsize, 0,
-                         size_t(P.ntiles) * 3 * h->np * TILE * h->rsize, h->stream));
-    }
-  }
-  return CMCG_OK;
+void set_source(cmcg_handle* h, const double* const* j_re, const double* const* j_im, int nused = -1) {
+  for (int p = 0; p < (nused < 0 ? h->nprob : nused); ++p)
+    source_to_int<R>(h, p, j_re[p], j_im ? j_im[p] : nullptr, h->J);
 }
 
 // Device status after a synchronised sweep: CMCG_ERR_DEVICE_TIMEOUT if a stage kernel's bounded
@@ -646,12 +656,11 @@ int check_err(cmcg_handle* h) {
 template <typename R>
 int forward_dev(cmcg_handle* h, const double* u0, const double* j_re, const double* j_im, double* uT, double* fre,
                 double* fim) {
-  for (int p = 0; p < nconv(h); ++p) to_int<R>(h, p, u0, 6, h->Uw, 6, 6, nullptr);
+  for (int p = 0; p < nconv(h); ++p) field_to_int<R>(h, p, u0, h->Uw);
   const bool filter = fre && fim;
   if (j_re) {
     std::vector<const double*> jr(size_t(h->nprob), j_re), ji(size_t(h->nprob), j_im);
-    int rc = set_source<R>(h, jr.data(), ji.data(), nconv(h));
-    if (rc) return rc;
+    set_source<R>(h, jr.data(), ji.data(), nconv(h));
   }
   if (filter) {
     CK(cudaMemsetAsync(h->Fre, 0, h->nvec * h->rsize, h->stream));
@@ -660,10 +669,10 @@ int forward_dev(cmcg_handle* h, const double* u0, const double* j_re, const doub
   if (j_re || filter) sweep_source<R>(h, j_re != nullptr, filter);
   else sweep_free<R>(h, false, nullptr);
   for (int p = 0; p < nconv(h); ++p) {
-    if (uT) to_ext<R>(h, p, h->Uw, 6, 0, uT, 6, 6);
+    if (uT) field_to_ext<R>(h, p, h->Uw, uT);
     if (filter) {
-      to_ext<R>(h, p, h->Fre, 6, 0, fre, 6, 6);
-      to_ext<R>(h, p, h->Fim, 6, 0, fim, 6, 6);
+      field_to_ext<R>(h, p, h->Fre, fre);
+      field_to_ext<R>(h, p, h->Fim, fim);
     }
   }
   CK(cudaGetLastError());
@@ -672,9 +681,9 @@ int forward_dev(cmcg_handle* h, const double* u0, const double* j_re, const doub
 
 template <typename R>
 int adjoint_dev(cmcg_handle* h, const double* wT, double* w0) {
-  for (int p = 0; p < nconv(h); ++p) to_int<R>(h, p, wT, 6, h->Uw, 6, 6, nullptr);
+  for (int p = 0; p < nconv(h); ++p) field_to_int<R>(h, p, wT, h->Uw);
   sweep_free<R>(h, true, nullptr);
-  for (int p = 0; p < nconv(h); ++p) to_ext<R>(h, p, h->Uw, 6, 0, w0, 6, 6);
+  for (int p = 0; p < nconv(h); ++p) field_to_ext<R>(h, p, h->Uw, w0);
   CK(cudaGetLastError());
   return check_err(h);
 }
@@ -682,7 +691,7 @@ int adjoint_dev(cmcg_handle* h, const double* wT, double* w0) {
 template <typename R>
 int apply_dev(cmcg_handle* h, double t, const double* u, const double* j_re, const double* j_im, int adjoint,
               double* out) {
-  for (int p = 0; p < nconv(h); ++p) to_int<R>(h, p, u, 6, h->Uw, 6, 6, nullptr);
+  for (int p = 0; p < nconv(h); ++p) field_to_int<R>(h, p, u, h->Uw);
   CK(cudaMemsetAsync(h->vB, 0, h->nvec * h->rsize, h->stream));
   StageCoef<R> c;
   std::memset(&c, 0, sizeof(c));
@@ -700,17 +709,15 @@ int apply_dev(cmcg_handle* h, double t, const double* u, const double* j_re, con
   a.coef = (const StageCoef<R>*)h->tab_one;
   if (j_re && !adjoint) {
     std::vector<const double*> jr(size_t(h->nprob), j_re), ji(size_t(h->nprob), j_im);
-    int rc = set_source<R>(h, jr.data(), ji.data(), nconv(h));
-    if (rc) return rc;
-    a.jre = (const R*)h->Jre;
-    a.jim = (const R*)h->Jim;
+    set_source<R>(h, jr.data(), ji.data(), nconv(h));
+    a.j = (const R*)h->J;
     if (h->has_bdata) {
       a.bre = (const R*)h->Bre;
       a.bim = (const R*)h->Bim;
     }
   }
   stage<R>(h, a);
-  for (int p = 0; p < nconv(h); ++p) to_ext<R>(h, p, h->vA, 6, 0, out, 6, 6);
+  for (int p = 0; p < nconv(h); ++p) field_to_ext<R>(h, p, h->vA, out);
   CK(cudaGetLastError());
   return check_err(h);
 }
@@ -718,8 +725,8 @@ int apply_dev(cmcg_handle* h, double t, const double* u, const double* j_re, con
 template <typename R>
 int inner_dev(cmcg_handle* h, const double* u, const double* v, double* out) {
   for (int p = 0; p < nconv(h); ++p) {
-    to_int<R>(h, p, u, 6, h->Uw, 6, 6, nullptr);
-    to_int<R>(h, p, v, 6, h->vA, 6, 6, nullptr);
+    field_to_int<R>(h, p, u, h->Uw);
+    field_to_int<R>(h, p, v, h->vA);
   }
   launch_dot<R>(h->q, (const R*)h->Uw, (const R*)h->vA, h->wdot, h->partials, h->bt, h->stream);
   launch_finalize(h->partials, h->bt, h->sc, nullptr, nullptr, 3, 0.0, h->stream);
@@ -759,20 +766,15 @@ int solve_dev(cmcg_handle* h, int nused, const double* const* j_re, const double
   for (int p = 0; p < h->nprob; ++p) h->used_host[p] = p < nused ? 1 : 0;
   CK(cudaMemcpyAsync(h->used, h->used_host, sizeof(int32_t) * h->nprob, cudaMemcpyHostToDevice, h->stream));
   const int32_t* mask = nused < h->nprob ? h->used : nullptr;
-  int rc = set_source<R>(h, j_re, j_im, nused);
-  if (rc) return rc;
+  set_source<R>(h, j_re, j_im, nused);
+  int rc = CMCG_OK;
   if ((rc = cg_phase<R>(h, mask, tol, max_iter))) return rc;
   // Final filter F_{psi,w} U0 for every used problem.
   lincomb<R>(h, h->Uw, nullptr, nullptr, 1.0, h->U0, 0.0, nullptr);
   CK(cudaMemsetAsync(h->Fre, 0, h->nvec * h->rsize, h->stream));
   CK(cudaMemsetAsync(h->Fim, 0, h->nvec * h->rsize, h->stream));
   sweep_source<R>(h, true, true, mask);
-  for (int p = 0; p < nused; ++p) {
-    to_ext<R>(h, p, h->Fre, 6, 0, e_re[p], 3, 3);
-    to_ext<R>(h, p, h->Fim, 6, 0, e_im[p], 3, 3);
-    to_ext<R>(h, p, h->Fre, 6, 3, h_re[p], 3, 3);
-    to_ext<R>(h, p, h->Fim, 6, 3, h_im[p], 3, 3);
-  }
+  for (int p = 0; p < nused; ++p) filtered_to_ext<R>(h, p, e_re[p], e_im[p], h_re[p], h_im[p]);
   CK(cudaEventRecord(ev1, h->stream));
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(h->stream));
@@ -870,18 +872,17 @@ int solve_multi_dev(cmcg_handle* h, int K, const int* harm, const double* const*
                     double tol, int max_iter, double* e_re, double* e_im, double* h_re, double* h_im, Sink&& sink,
                     cmcg_info* info) {
   Prob& P = h->P[0];
-  const size_t vb = size_t(h->njvec) * h->rsize;
+  const size_t vb = size_t(h->nvec) * h->rsize;
   if (K > h->mf_cap) {  // K sources and the per-launch harmonic coefficients (kept for later calls)
-    if (h->Jm_re) cudaFree(h->Jm_re);
-    if (h->Jm_im) cudaFree(h->Jm_im);
+    if (h->Jm) cudaFree(h->Jm);
     if (h->mf_hcs) cudaFree(h->mf_hcs);
-    h->Jm_re = h->Jm_im = h->mf_hcs = nullptr;
+    h->Jm = h->mf_hcs = nullptr;
     h->mf_cap = 0;
-    if (cudaMalloc(&h->Jm_re, vb * K) != cudaSuccess || cudaMalloc(&h->Jm_im, vb * K) != cudaSuccess ||
+    if (cudaMalloc(&h->Jm, vb * K) != cudaSuccess ||
         cudaMalloc(&h->mf_hcs, size_t(h->L_srcf) * 2 * K * h->rsize) != cudaSuccess)
       return CMCG_ERR_OUT_OF_MEMORY;
     h->mf_cap = K;
-    h->bytes += 2 * vb * K + size_t(h->L_srcf) * 2 * K * h->rsize;
+    h->bytes += vb * K + size_t(h->L_srcf) * 2 * K * h->rsize;
   }
   if (!h->mf_tab) {
     if (cudaMalloc(&h->mf_tab, size_t(h->L_srcf) * sizeof(StageCoef<R>)) != cudaSuccess) return CMCG_ERR_OUT_OF_MEMORY;
@@ -904,13 +905,8 @@ int solve_multi_dev(cmcg_handle* h, int K, const int* harm, const double* const*
   CK(cudaEventCreate(&ev0));
   CK(cudaEventCreate(&ev1));
   CK(cudaEventRecord(ev0, h->stream));
-  for (int k = 0; k < K; ++k) {
-    void* jr = static_cast<char*>(h->Jm_re) + vb * k;
-    void* ji = static_cast<char*>(h->Jm_im) + vb * k;
-    to_int<R>(h, 0, j_re[k], 3, jr, 3, 3, h->inv_eps);
-    if (j_im && j_im[k]) to_int<R>(h, 0, j_im[k], 3, ji, 3, 3, h->inv_eps);
-    else CK(cudaMemsetAsync(ji, 0, vb, h->stream));
-  }
+  for (int k = 0; k < K; ++k)
+    source_to_int<R>(h, 0, j_re[k], j_im ? j_im[k] : nullptr, static_cast<char*>(h->Jm) + vb * k);
   h->used_host[0] = 1;  // the problem takes part (read by the first reduction of the CG phase)
   CK(cudaMemcpyAsync(h->used, h->used_host, sizeof(int32_t), cudaMemcpyHostToDevice, h->stream));
   h->mf_nharm = K;
@@ -942,10 +938,7 @@ int solve_multi_dev(cmcg_handle* h, int K, const int* harm, const double* const*
     CK(cudaMemsetAsync(h->Fre, 0, h->nvec * h->rsize, h->stream));
     CK(cudaMemsetAsync(h->Fim, 0, h->nvec * h->rsize, h->stream));
     sweep_source<R>(h, true, true, nullptr);
-    to_ext<R>(h, 0, h->Fre, 6, 0, e_re, 3, 3);
-    to_ext<R>(h, 0, h->Fim, 6, 0, e_im, 3, 3);
-    to_ext<R>(h, 0, h->Fre, 6, 3, h_re, 3, 3);
-    to_ext<R>(h, 0, h->Fim, 6, 3, h_im, 3, 3);
+    filtered_to_ext<R>(h, 0, e_re, e_im, h_re, h_im);
     rc = sink(k);
     CK(cudaStreamSynchronize(h->stream));  // the host filter table is rebuilt for the next harmonic
   }
@@ -1066,10 +1059,7 @@ int slot_round_dev(cmcg_handle* h, double tol, int max_iter, int* done) {
     for (int p = 0; p < n; ++p)
       if (mh[2 * n + p]) {
         const size_t off = size_t(h->P[size_t(p)].ext0) * 3 * h->np;
-        to_ext<R>(h, p, h->Fre, 6, 0, h->ext0 + off, 3, 3);
-        to_ext<R>(h, p, h->Fim, 6, 0, h->ext0 + half + off, 3, 3);
-        to_ext<R>(h, p, h->Fre, 6, 3, h->ext1 + off, 3, 3);
-        to_ext<R>(h, p, h->Fim, 6, 3, h->ext1 + half + off, 3, 3);
+        filtered_to_ext<R>(h, p, h->ext0 + off, h->ext0 + half + off, h->ext1 + off, h->ext1 + half + off);
       }
   }
   CK(cudaGetLastError());
@@ -1117,8 +1107,7 @@ int slot_round_dev(cmcg_handle* h, double tol, int max_iter, int* done) {
 template <typename R>
 int fw_dev(cmcg_handle* h, int periods, const double* const* j_re, const double* const* j_im, double* const* e_re,
            double* const* e_im, double* const* h_re, double* const* h_im) {
-  int rc = set_source<R>(h, j_re, j_im, h->nprob);
-  if (rc) return rc;
+  set_source<R>(h, j_re, j_im, h->nprob);
   CK(cudaMemsetAsync(h->Uw, 0, h->nvec * h->rsize, h->stream));
   if (periods > 0) sweep_source<R>(h, true, false, nullptr);
   if (periods > 1) lincomb<R>(h, h->A, nullptr, nullptr, 1.0, h->Uw, 0.0, nullptr);
@@ -1129,12 +1118,7 @@ int fw_dev(cmcg_handle* h, int periods, const double* const* j_re, const double*
   CK(cudaMemsetAsync(h->Fre, 0, h->nvec * h->rsize, h->stream));
   CK(cudaMemsetAsync(h->Fim, 0, h->nvec * h->rsize, h->stream));
   sweep_source<R>(h, true, true, nullptr);
-  for (int p = 0; p < h->nprob; ++p) {
-    to_ext<R>(h, p, h->Fre, 6, 0, e_re[p], 3, 3);
-    to_ext<R>(h, p, h->Fim, 6, 0, e_im[p], 3, 3);
-    to_ext<R>(h, p, h->Fre, 6, 3, h_re[p], 3, 3);
-    to_ext<R>(h, p, h->Fim, 6, 3, h_im[p], 3, 3);
-  }
+  for (int p = 0; p < h->nprob; ++p) filtered_to_ext<R>(h, p, e_re[p], e_im[p], h_re[p], h_im[p]);
   CK(cudaGetLastError());
   return check_err(h);
 }
@@ -1150,10 +1134,10 @@ void free_all(cmcg_handle* h) {
   drop_graphs(h);
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   h->cap_stream = nullptr;
-  void* ptrs[] = {h->Jm_re, h->Jm_im, h->mf_hcs, h->mf_tab, h->mf_src,
-                  h->gvol, h->gface, h->nbr, h->wdot, h->e_of_i, h->tprob, h->inv_eps, h->Uw, h->vA, h->vB,
-                  h->Fre, h->Fim, h->Jre, h->Jim, h->Bre, h->Bim, h->U0, h->Rv, h->D, h->A, h->WT, h->partials, h->sc, h->pactive,
-                  h->bt_tet0, h->bt_ntet, h->bt_prob, h->bt_pb0, h->tab_free, h->tab_src, h->tab_srcf, h->tab_one,
+  void* ptrs[] = {h->Jm, h->mf_hcs, h->mf_tab, h->mf_src,
+                  h->geo, h->nbr, h->wdot, h->e_of_i, h->tprob, h->inv_eps, h->Uw, h->vA, h->vB,
+                  h->Fre, h->Fim, h->J, h->Bre, h->Bim, h->U0, h->Rv, h->D, h->A, h->WT, h->partials, h->sc, h->pactive,
+                  h->bt_half, h->bt_tet0, h->bt_ntet, h->bt_prob, h->bt_pb0, h->tab_free, h->tab_src, h->tab_srcf, h->tab_one,
                   h->ext0, h->ext1, h->ext2, h->ext3, h->used, h->err, h->slot_masks, h->halo_dst, h->halo_src, h->g_in,
                   h->g_out, h->inv_eps_g};
   for (void* p : ptrs)
@@ -1201,8 +1185,8 @@ int create_impl(int nprob, const cmcg_problem* probs, const cmcg_options* opt_in
   h->rsize = opt.precision == CMCG_FP32 ? 4 : 8;
   h->P.resize(nprob);
   // Host layouts, concatenated.
-  std::vector<double> gvol, gface, wdot, inv_eps;
-  std::vector<int32_t> nbr, e_of_i, tprob;
+  std::vector<double> geo, wdot, inv_eps;
+  std::vector<int32_t> nbr, e_of_i, tprob, half_at;
   int rc = CMCG_OK;
   try {
     for (int p = 0; p < nprob && rc == CMCG_OK; ++p) {
@@ -1227,28 +1211,17 @@ int create_impl(int nprob, const cmcg_problem* probs, const cmcg_options* opt_in
         rc = CMCG_ERR_INVALID_ARG;
         break;
       }
-      gvol.insert(gvol.end(), L.gvol.begin(), L.gvol.end());
-      gface.insert(gface.end(), L.gface.begin(), L.gface.end());
+      geo.insert(geo.end(), L.geo.begin(), L.geo.end());
       wdot.insert(wdot.end(), L.wdot.begin(), L.wdot.end());
       const int32_t shift = int32_t(P.tet0) << 5;
-      for (int32_t c : L.nbr) nbr.push_back(c >= 0 ? c + shift : c);
-      for (int64_t t = 0; t < L.ntiles; ++t)
-        for (int f = 0; f < 4; ++f)
-          for (int l = 0; l < TILE; ++l) {
-            if (L.nbr[(t * 4 + f) * TILE + l] != NBR_IMP || L.ext_of_int[t * TILE + l] < 0) continue;
-            ImpFace F;
-            F.it = P.tet0 + t * TILE + l;
-            F.ext = L.ext_of_int[t * TILE + l];
-            F.f = f;
-            auto gf = [&](int item) { return L.gface[((t * 4 + f) * GF + item) * TILE + l]; };
-            for (int a = 0; a < 3; ++a) F.n[a] = gf(a);
-            F.bH = gf(3);
-            F.aE = gf(6);
-            P.imp.push_back(F);
-          }
+      for (int32_t c : L.nbr) nbr.push_back(c + shift);
+      P.imp = L.imp;
+      for (ImpFace& F : P.imp) F.it += P.tet0;
       e_of_i.insert(e_of_i.end(), L.ext_of_int.begin(), L.ext_of_int.end());
       P.ext_of_int = L.ext_of_int;
       P.int_of_ext = L.int_of_ext;
+      P.half_at = L.half_at;
+      for (int32_t x : L.half_at) half_at.push_back(x + int32_t(P.tet0 / HTILE));
       for (int64_t t = 0; t < L.ntiles; ++t) tprob.push_back(p);
       for (int64_t k = 0; k < L.nt; ++k) inv_eps.push_back(1.0 / probs[p].eps[k]);
       h->nti += L.nti;
@@ -1266,24 +1239,22 @@ int create_impl(int nprob, const cmcg_problem* probs, const cmcg_options* opt_in
   }
   h->np = np_of(h->q);
   h->nvec = h->nti * 6 * h->np;
-  h->njvec = h->nti * 3 * h->np;
   // Problem-aligned reduction blocks.
   std::vector<int64_t> bt_tet0;
   std::vector<int32_t> bt_ntet, bt_prob, bt_pb0;
   for (int p = 0; p < nprob; ++p) {
     bt_pb0.push_back(int32_t(bt_tet0.size()));
-    for (int64_t t = 0; t < h->P[p].nti; t += DOT_THREADS) {
+    for (int64_t t = 0; t < h->P[p].nti; t += DOT_TETS) {
       bt_tet0.push_back(h->P[p].tet0 + t);
-      bt_ntet.push_back(int32_t(std::min<int64_t>(DOT_THREADS, h->P[p].nti - t)));
+      bt_ntet.push_back(int32_t(std::min<int64_t>(DOT_TETS, h->P[p].nti - t)));
       bt_prob.push_back(p);
     }
   }
   bt_pb0.push_back(int32_t(bt_tet0.size()));
 
   const size_t extlen = size_t(h->nt_total) * 6 * h->np * sizeof(double);
-  const size_t need = 11 * h->nvec * h->rsize + 2 * h->njvec * h->rsize + gvol.size() * h->rsize +
-                      gface.size() * h->rsize + nbr.size() * 4 + wdot.size() * 8 + e_of_i.size() * 4 +
-                      inv_eps.size() * 8 + 4 * extlen + bt_tet0.size() * 24 + size_t(nprob) * 128 +
+  const size_t need = 12 * h->nvec * h->rsize + geo.size() * h->rsize + nbr.size() * 4 + wdot.size() * 8 + e_of_i.size() * 4 +
+                      inv_eps.size() * 8 + 4 * extlen + half_at.size() * 4 + bt_tet0.size() * 24 + size_t(nprob) * 128 +
                       size_t(3 * h->maxM * h->s + 2) * nprob * sizeof(StageCoef<double>);
   h->bytes = need;
   if (opt.hbm_budget_bytes > 0 && (int64_t)need > opt.hbm_budget_bytes) {
@@ -1312,23 +1283,22 @@ int create_impl(int nprob, const cmcg_problem* probs, const cmcg_options* opt_in
 
   size_t bytes = 0;
   if (h->prec == CMCG_FP32) {
-    if ((rc = upload(&h->gvol, cast<float>(gvol), &bytes)) || (rc = upload(&h->gface, cast<float>(gface), &bytes)))
-      return fail(rc);
+    if ((rc = upload(&h->geo, cast<float>(geo), &bytes))) return fail(rc);
   } else {
-    if ((rc = upload(&h->gvol, gvol, &bytes)) || (rc = upload(&h->gface, gface, &bytes))) return fail(rc);
+    if ((rc = upload(&h->geo, geo, &bytes))) return fail(rc);
   }
   if ((rc = upload((void**)&h->nbr, nbr, &bytes)) || (rc = upload((void**)&h->wdot, wdot, &bytes)) ||
       (rc = upload((void**)&h->e_of_i, e_of_i, &bytes)) || (rc = upload((void**)&h->inv_eps, inv_eps, &bytes)) ||
-      (rc = upload((void**)&h->bt_tet0, bt_tet0, &bytes)) || (rc = upload((void**)&h->bt_ntet, bt_ntet, &bytes)) ||
+      (rc = upload((void**)&h->bt_half, half_at, &bytes)) || (rc = upload((void**)&h->bt_tet0, bt_tet0, &bytes)) || (rc = upload((void**)&h->bt_ntet, bt_ntet, &bytes)) ||
       (rc = upload((void**)&h->bt_prob, bt_prob, &bytes)) || (rc = upload((void**)&h->bt_pb0, bt_pb0, &bytes)))
     return fail(rc);
   if (nprob > 1 && (rc = upload((void**)&h->tprob, tprob, &bytes))) return fail(rc);
-  h->bt = BlockTable{h->bt_tet0, h->bt_ntet, h->bt_prob, h->bt_pb0, int(bt_tet0.size()), nprob};
+  h->bt = BlockTable{h->bt_half, h->bt_tet0, h->bt_ntet, h->bt_prob, h->bt_pb0, int(bt_tet0.size()), nprob};
 
   auto alloc = [&](void** p, size_t n) -> bool { return cudaMalloc(p, n) == cudaSuccess; };
-  const size_t vb = h->nvec * h->rsize, jb = h->njvec * h->rsize;
+  const size_t vb = h->nvec * h->rsize;
   bool ok = alloc(&h->Uw, vb) && alloc(&h->vA, vb) && alloc(&h->vB, vb) && alloc(&h->Fre, vb) &&
-            alloc(&h->Fim, vb) && alloc(&h->Jre, jb) && alloc(&h->Jim, jb) && alloc(&h->U0, vb) &&
+            alloc(&h->Fim, vb) && alloc(&h->J, vb) && alloc(&h->U0, vb) &&
             alloc(&h->Rv, vb) && alloc(&h->D, vb) && alloc(&h->A, vb) && alloc(&h->WT, vb) &&
             alloc((void**)&h->partials, sizeof(double) * 2 * std::max<size_t>(1, bt_tet0.size())) &&
             alloc((void**)&h->sc, sizeof(Scalars) * nprob) && alloc((void**)&h->pactive, sizeof(int32_t) * nprob) &&
@@ -1351,8 +1321,12 @@ int create_impl(int nprob, const cmcg_problem* probs, const cmcg_options* opt_in
     h->form = opt.stage_variant - 1;
     h->pdl = opt.stage_overlap != 2;
   } else {
-    rc = h->prec == CMCG_FP32 ? autotune<float>(h, STAGE_FORMS_F32, opt.stage_overlap)
-                              : autotune<double>(h, STAGE_FORMS_F64, opt.stage_overlap);
+    // P3 in FP32 always takes the tensor-core form (16.5 us per stage of 12,288 tetrahedra against 27 for
+    // the best other one, 37 against 95 at 48,000), P1 and P2 one of the others (P2: 22 us against 31
+    // at 81,648 tetrahedra): the arithmetic does not depend on what was measured.
+    if (h->prec == CMCG_FP64) rc = autotune<double>(h, 0, STAGE_FORMS_F64, opt.stage_overlap);
+    else if (h->q == 3) rc = autotune<float>(h, STAGE_FORM_TC, 1, opt.stage_overlap);
+    else rc = autotune<float>(h, 0, STAGE_FORM_TC, opt.stage_overlap);
     if (rc) return fail(rc);
   }
   h->graphs = opt.launch_graphs != 2;
@@ -1858,6 +1832,10 @@ int cmcg_set_boundary_data(cmcg_handle* h, int problem, const double* g_re, cons
         }
       }
     }
+    if (h->prec == CMCG_FP64) {  // the nodal values of 6 components per tetrahedron
+      to_bern_rows(h->q, hre);
+      to_bern_rows(h->q, him);
+    }
     CK(cudaMemsetAsync(static_cast<char*>(h->Bre) + off * R_, 0, cnt * R_, h->stream));
     CK(cudaMemsetAsync(static_cast<char*>(h->Bim) + off * R_, 0, cnt * R_, h->stream));
     if (!tets.empty()) {
@@ -1923,11 +1901,11 @@ int cmcg_set_conductivity(cmcg_handle* h, int problem, const double* sigma) {
   } else {
     CK(cudaMemsetAsync(dsig, 0, size_t(P.nt) * sizeof(double), h->stream));
   }
-  void* gv = static_cast<char*>(h->gvol) + size_t(P.tile0) * GV * TILE * h->rsize;
+  void* geo = static_cast<char*>(h->geo) + size_t(P.tet0 / HTILE) * (h->prec == CMCG_FP32 ? GEO32 : GEO64) * h->rsize;
   if (h->prec == CMCG_FP32)
-    launch_set_gvol_item<float>((float*)gv, 11, dsig, h->inv_eps + P.ext0, h->e_of_i + P.tet0, P.nti, h->stream);
+    launch_set_sigma<float>((float*)geo, dsig, h->inv_eps + P.ext0, h->e_of_i + P.tet0, P.nti, h->stream);
   else
-    launch_set_gvol_item<double>((double*)gv, 11, dsig, h->inv_eps + P.ext0, h->e_of_i + P.tet0, P.nti, h->stream);
+    launch_set_sigma<double>((double*)geo, dsig, h->inv_eps + P.ext0, h->e_of_i + P.tet0, P.nti, h->stream);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(h->stream));
   P.has_sigma = sigma != nullptr;
@@ -1990,18 +1968,8 @@ int cmcg_slot_admit(cmcg_handle* h, int slot, const double* j_re, const double* 
     CK(cudaMemcpyAsync(h->ext3 + half + off, j_im, cnt * 8, cudaMemcpyHostToDevice, h->stream));
     ji = h->ext3 + half + off;
   }
-  if (h->prec == CMCG_FP32) {
-    to_int<float>(h, slot, jr, 3, h->Jre, 3, 3, h->inv_eps);
-    if (ji) to_int<float>(h, slot, ji, 3, h->Jim, 3, 3, h->inv_eps);
-  } else {
-    to_int<double>(h, slot, jr, 3, h->Jre, 3, 3, h->inv_eps);
-    if (ji) to_int<double>(h, slot, ji, 3, h->Jim, 3, 3, h->inv_eps);
-  }
-  if (!ji) {
-    const size_t per_tile = size_t(3) * h->np * TILE * h->rsize;
-    CK(cudaMemsetAsync(static_cast<char*>(h->Jim) + size_t(P.tile0) * per_tile, 0, size_t(P.ntiles) * per_tile,
-                       h->stream));
-  }
+  if (h->prec == CMCG_FP32) source_to_int<float>(h, slot, jr, ji, h->J);
+  else source_to_int<double>(h, slot, jr, ji, h->J);
   CK(cudaGetLastError());
   CK(cudaStreamSynchronize(h->stream));  // the host source may be reused when this returns
   h->slot_phase[size_t(slot)] = SLOT_ADMITTED;
@@ -2042,9 +2010,11 @@ int cmcg_slot_take(cmcg_handle* h, int slot, double* e_re, double* e_im, double*
 namespace {
 
 // Saved state of a slot (checkpoint between rounds): a header, then the problem's tiles of U0, R,
-// D (6 Np values per tetrahedron each) and of the source J_re, J_im (3 Np each), in the handle's
-// precision and internal layout.  Between rounds Uw holds D for an iterating slot; A and W_T are
-// scratch of a round.  Restoring it gives the same bits as never having stopped.
+// D and of the source J (6 Np values per tetrahedron each), in the handle's precision, basis and
+// layout.  Between rounds Uw holds D for an iterating slot; A and W_T are scratch of a round.
+// Restoring it gives the same bits as never having stopped.  States of the first format (nodal
+// values, [tile][component][node][32] in the order of the shape classes, J_re and J_im apart) are
+// accepted and converted.
 struct SlotHeader {
   char magic[8];
   int32_t prec, q, np, M, phase, pactive;
@@ -2052,11 +2022,35 @@ struct SlotHeader {
   double dt, omega;
   Scalars sc;
 };
-constexpr char SLOT_MAGIC[8] = {'C', 'M', 'C', 'G', 'S', 'L', 'T', '1'};
+constexpr char SLOT_MAGIC[8] = {'C', 'M', 'C', 'G', 'S', 'L', 'T', '2'};
+constexpr char SLOT_MAGIC1[8] = {'C', 'M', 'C', 'G', 'S', 'L', 'T', '1'};
+
+// The payload of a state of the first format in the present one.
+template <typename R>
+void slot_from_first(const cmcg_handle* h, const Prob& P, const R* in, R* out) {
+  const int np = h->np;
+  const size_t v6 = size_t(P.ntiles) * TILE * 6 * np;
+  std::vector<R> u(static_cast<size_t>(np));
+  for (int64_t t = 0; t < P.ntiles; ++t)
+    for (int l = 0; l < TILE; ++l)
+      for (int vec = 0; vec < 4; ++vec)  // U0, R, D, J
+        for (int f = 0; f < 2; ++f)
+          for (int c = 0; c < 3; ++c) {
+            const size_t tile = size_t(t);
+            const R* src = vec < 3 ? in + vec * v6 + (tile * 6 + 3 * f + c) * np * TILE
+                                   : in + 3 * v6 + f * (v6 / 2) + (tile * 3 + c) * np * TILE;
+            for (int n = 0; n < np; ++n) u[n] = src[n * TILE + l];
+            if (h->prec == CMCG_FP64) to_bern_rows(h->q, u);
+            for (int n = 0; n < np; ++n) {
+              const int64_t i = int64_t(P.half_at[size_t(2 * t + l / HTILE)]) * HTILE + l % HTILE;
+              out[vec * v6 + size_t(field_at(np, i, f, c, n))] = u[n];
+            }
+          }
+}
 
 size_t slot_payload(const cmcg_handle* h, int slot) {
   const Prob& P = h->P[size_t(slot)];
-  return size_t(P.ntiles) * TILE * h->np * h->rsize * (3 * 6 + 2 * 3);
+  return size_t(P.ntiles) * TILE * h->np * h->rsize * (4 * 6);
 }
 
 }  // namespace
@@ -2091,14 +2085,11 @@ int cmcg_slot_save(cmcg_handle* h, int slot, void* buf, int64_t len) {
   CK(cudaMemcpyAsync(&hd.sc, h->sc + slot, sizeof(Scalars), cudaMemcpyDeviceToHost, h->stream));
   CK(cudaMemcpyAsync(&hd.pactive, h->pactive + slot, sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream));
   char* out = static_cast<char*>(buf) + sizeof(SlotHeader);
-  const size_t v6 = size_t(P.ntiles) * 6 * h->np * TILE * h->rsize, v3 = v6 / 2;
-  const size_t o6 = size_t(P.tile0) * 6 * h->np * TILE * h->rsize, o3 = o6 / 2;
-  const void* src6[3] = {h->U0, h->Rv, h->D};
-  for (int k = 0; k < 3; ++k, out += v6)
+  const size_t v6 = size_t(P.ntiles) * 6 * h->np * TILE * h->rsize;
+  const size_t o6 = size_t(P.tile0) * 6 * h->np * TILE * h->rsize;
+  const void* src6[4] = {h->U0, h->Rv, h->D, h->J};
+  for (int k = 0; k < 4; ++k, out += v6)
     CK(cudaMemcpyAsync(out, static_cast<const char*>(src6[k]) + o6, v6, cudaMemcpyDeviceToHost, h->stream));
-  const void* src3[2] = {h->Jre, h->Jim};
-  for (int k = 0; k < 2; ++k, out += v3)
-    CK(cudaMemcpyAsync(out, static_cast<const char*>(src3[k]) + o3, v3, cudaMemcpyDeviceToHost, h->stream));
   const int32_t zero = 0;
   CK(cudaMemcpyAsync(h->pactive + slot, &zero, sizeof(int32_t), cudaMemcpyHostToDevice, h->stream));
   CK(cudaStreamSynchronize(h->stream));
@@ -2114,7 +2105,8 @@ int cmcg_slot_restore(cmcg_handle* h, int slot, const void* buf, int64_t len) {
   SlotHeader hd;
   std::memcpy(&hd, buf, sizeof(hd));
   const Prob& P = h->P[size_t(slot)];
-  if (std::memcmp(hd.magic, SLOT_MAGIC, 8) != 0 || hd.prec != h->prec || hd.q != h->q || hd.np != h->np ||
+  const bool first = std::memcmp(hd.magic, SLOT_MAGIC1, 8) == 0;
+  if ((!first && std::memcmp(hd.magic, SLOT_MAGIC, 8) != 0) || hd.prec != h->prec || hd.q != h->q || hd.np != h->np ||
       hd.M != P.M || hd.nt != P.nt || hd.ntiles != P.ntiles || hd.dt != P.dt || hd.omega != P.omega ||
       (hd.phase != SLOT_ADMITTED && hd.phase != SLOT_CG && hd.phase != SLOT_FINAL) ||
       len < int64_t(sizeof(SlotHeader) + slot_payload(h, slot)))
@@ -2124,14 +2116,22 @@ int cmcg_slot_restore(cmcg_handle* h, int slot, const void* buf, int64_t len) {
   if (rc) return rc;
   if (h->slot_phase[size_t(slot)] != SLOT_EMPTY) return CMCG_ERR_INVALID_ARG;
   const char* in = static_cast<const char*>(buf) + sizeof(SlotHeader);
-  const size_t v6 = size_t(P.ntiles) * 6 * h->np * TILE * h->rsize, v3 = v6 / 2;
-  const size_t o6 = size_t(P.tile0) * 6 * h->np * TILE * h->rsize, o3 = o6 / 2;
-  void* dst6[3] = {h->U0, h->Rv, h->D};
-  for (int k = 0; k < 3; ++k, in += v6)
+  std::vector<char> conv;
+  if (first) {
+    try {
+      conv.resize(slot_payload(h, slot));
+      if (h->prec == CMCG_FP32) slot_from_first(h, P, reinterpret_cast<const float*>(in), reinterpret_cast<float*>(conv.data()));
+      else slot_from_first(h, P, reinterpret_cast<const double*>(in), reinterpret_cast<double*>(conv.data()));
+    } catch (const std::bad_alloc&) {
+      return CMCG_ERR_OUT_OF_MEMORY;
+    }
+    in = conv.data();
+  }
+  const size_t v6 = size_t(P.ntiles) * 6 * h->np * TILE * h->rsize;
+  const size_t o6 = size_t(P.tile0) * 6 * h->np * TILE * h->rsize;
+  void* dst6[4] = {h->U0, h->Rv, h->D, h->J};
+  for (int k = 0; k < 4; ++k, in += v6)
     CK(cudaMemcpyAsync(static_cast<char*>(dst6[k]) + o6, in, v6, cudaMemcpyHostToDevice, h->stream));
-  void* dst3[2] = {h->Jre, h->Jim};
-  for (int k = 0; k < 2; ++k, in += v3)
-    CK(cudaMemcpyAsync(static_cast<char*>(dst3[k]) + o3, in, v3, cudaMemcpyHostToDevice, h->stream));
   // an iterating slot starts its next round with Uw = D
   CK(cudaMemcpyAsync(static_cast<char*>(h->Uw) + o6, static_cast<const char*>(h->D) + o6, v6,
                      cudaMemcpyDeviceToDevice, h->stream));

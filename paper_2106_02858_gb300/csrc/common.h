@@ -61,9 +61,19 @@ struct RefMats {
   std::vector<double> LIFT;                 // np x (4 nfp), face-local node order
   std::vector<int> fmask;                   // 4 x nfp
   std::vector<int> nbrnode;                 // 4 (neighbour face) x 6 (perm) x nfp
+
   double face_ref_area[4] = {0, 0, 0, 0};
 };
 const RefMats& ref_mats(int q);
+
+// An impedance face: what its boundary data need on the host.
+struct ImpFace {
+  int64_t it = 0;        // internal tetrahedron
+  int32_t ext = 0;       // external tetrahedron within its problem
+  int f = 0;             // face
+  double n[3] = {0, 0, 0};
+  double aE = 0, bH = 0;  // flux coefficients of the E rows (tangential jump) and H rows (n x jump)
+};
 
 // Per-tetrahedron geometry in the device layout, built on the host.
 struct HostLayout {
@@ -71,16 +81,26 @@ struct HostLayout {
   int64_t nt = 0, nti = 0, ntiles = 0;
   std::vector<int32_t> ext_of_int;  // internal -> external tet (-1 = padding)
   std::vector<int32_t> int_of_ext;  // external -> internal
-  std::vector<double> gvol;         // [tile][GV][32]
-  std::vector<double> gface;        // [tile][4][GF][32]
-  std::vector<int32_t> nbr;         // [tile][4][32]
-  std::vector<double> wdot;         // [tile][2][32]: |det| eps, |det| mu
+  std::vector<int32_t> half_at;     // half tile in the order of the shape classes -> internal half tile
+  std::vector<double> geo;          // [half tile][GEO32 or GEO64]
+  std::vector<int32_t> nbr;         // [half tile][4][16]
+  std::vector<double> wdot;         // [half tile][16][2]: |det| eps, |det| mu
+  std::vector<ImpFace> imp;         // impedance faces (internal tetrahedra of this layout)
   int steps = 0;
   double dt = 0, T = 0, rho_min = 0;
   int ngroups = 0;
 };
-constexpr int GV = 12;  // G (9, d r_b / d x_a at [b*3+a]), 1/eps, 1/mu, sigma/eps (0 unless set)
-constexpr int GF = 8;   // nx, ny, nz, bH, aH, -bE, aE, pad  (see setup.cpp)
+// Geometry of a half tile (16 tetrahedra): items of 16 values that the two threads of a tetrahedron
+// share, G (9, d r_b / d x_a at [b*3+a]) and per face its outward normal (FP32) or a tangent frame
+// t1, t2 with t1 x t2 the outward normal (FP64); then GEO_P items of 32 values, one per thread
+// (even: computes Phi_H, odd: Phi_E): 1/mu | -1/eps, per face k1 and k2 (FP32; bH, aH | -bE, aE) or
+// k1 and k2 / k1 (FP64), and sigma/eps (0 unless set).
+constexpr int GEO_S32 = 9 + 4 * 3;
+constexpr int GEO_S64 = 9 + 4 * 6;
+constexpr int GEO_P = 1 + 4 * 2 + 1;
+constexpr int GEO_SIGMA = 9;  // per-thread item of sigma/eps
+constexpr int GEO32 = GEO_S32 * 16 + GEO_P * 32;
+constexpr int GEO64 = GEO_S64 * 16 + GEO_P * 32;
 
 int validate_and_layout(const cmcg_mesh* mesh, const double* eps, const double* mu, double omega,
                         const cmcg_options* opt, HostLayout* out, bool build_layout, std::string* why);
@@ -103,13 +123,14 @@ struct ShardPlan {
 int shard_plan(const cmcg_mesh* mesh, const std::vector<int64_t>& nb, const int32_t* part, int nparts, int p,
                ShardPlan* out);
 
-// Neighbour code: >= 0: (internal neighbour << 5) | (neighbour face << 3) | perm.
-constexpr int32_t NBR_PEC = -1;
-constexpr int32_t NBR_IMP = -2;
+// Neighbour code: (internal neighbour << 5) | (neighbour face << 3) | perm.  A boundary face names
+// its own tetrahedron and face, with perm PERM_PEC or PERM_IMP (the identity permutation).
+constexpr int32_t PERM_PEC = 6;
+constexpr int32_t PERM_IMP = 7;
 
 // Per-problem coefficients of one stage launch (a handle holds a batch of
 // problems that advance in lockstep; each reads its own entry).
-//   Phi   = src + B_sigma(vin),  src = s_cos * (jre + bre) - s_sin * (jim + bim)   (B_sigma = Sigma B Sigma when sH = -1;
+//   Phi   = src + B_sigma(vin),  src = s_cos * (J_re + bre) - s_sin * (J_im + bim)   (B_sigma = Sigma B Sigma when sH = -1;
 //           B carries -(sigma/eps) E on the E rows when a.sigma is set)
 //   out   = base + c_out Phi        (skipped if out == nullptr)
 //   F    += fa vin + fb Phi         (complex weights; skipped if fre == nullptr)
@@ -128,8 +149,8 @@ struct StageArgs {
   const R* vin;
   const R* base;
   R* out;
-  const R* jre;  // E-rows source / eps, [tile][3][Np][32] (null: no source)
-  const R* jim;
+  const R* j;    // E-rows source / eps in the field layout, J_re at the electric and J_im at the
+                 // magnetic places (null: no source)
   const R* bre;  // lifted impedance-face data, all 6 rows in the field layout (null: none)
   const R* bim;
   R* fre;        // filter accumulators (null: no filter)
@@ -138,25 +159,23 @@ struct StageArgs {
   const StageCoef<R>* coef;  // [problem] for this launch
   const int32_t* tprob;      // problem of each tile (null: every tile is problem 0)
   const int32_t* pactive;    // per-problem CG activity (null: all active)
-  const R* gvol;
-  const R* gface;
+  const R* geo;
   const int32_t* nbr;
   int64_t nti;
   int32_t* err;  // device status word: a stage kernel whose bounded wait ran out ORs in 1 (null: not recorded)
-  int32_t sigma;  // nonzero: some tetrahedron has a conductivity (sigma/eps in gvol item 11)
+  int32_t sigma;  // nonzero: some tetrahedron has a conductivity
   // Several harmonics in one sweep (nharm > 0): the source is sum_h hcs[2h] J_re,h - hcs[2h+1] J_im,h
-  // with J_h = jre / jim + h * jstride (hcs: this launch's cos / sin of the harmonics at the stage time).
+  // with J_h = j + h * jstride (hcs: this launch's cos / sin of the harmonics at the stage time).
   int32_t nharm;
   int64_t jstride;
   const R* hcs;
 };
 
 // Kernel launchers, one translation unit per order.
-// form: stage-kernel form.  FP32: 0, 1, 2 = two threads per tetrahedron with at
-// least 1, 3, 4 resident 128-thread blocks per SM; 3, 4, 5 = four threads per
-// tetrahedron with at least 4, 5, 6; 6 = tensor-core contractions (tcgen05,
-// 3xTF32) with two threads per tetrahedron.  FP64: 0 = two threads per
-// tetrahedron, 1, 2 = four threads per tetrahedron with at least 2, 3 blocks.
+// form: stage-kernel form.  FP32: 0, 1, 2 = one warp per half tile (two threads per
+// tetrahedron) with at least 3, 4, 6 resident 128-thread blocks per SM; 3, 4 = two warps
+// per half tile with at least 3, 4 blocks; 5 = four warps per half tile; 6 = tensor-core
+// contractions (tcgen05, 3xTF32).  FP64: 0, 1, 2 = one, two, four warps per half tile.
 // pdl: launch with programmatic stream serialisation (the stage overlaps the
 // previous stage's tail).
 constexpr int STAGE_FORMS_F32 = 7;
@@ -174,10 +193,11 @@ struct Scalars {
   int iters;
 };
 
-// Blocks of the problem-aligned reductions: block b covers internal tets
-// [tet0[b], tet0[b] + ntet[b]) of problem prob[b]; problem p owns blocks
-// [pb0[p], pb0[p + 1]).
+// Blocks of the problem-aligned reductions: block b covers tets [tet0[b], tet0[b] + ntet[b]) of
+// problem prob[b] in the order of the shape classes (half tile h of that order is internal half
+// tile half_at[h]); problem p owns blocks [pb0[p], pb0[p + 1]).
 struct BlockTable {
+  const int32_t* half_at;
   const int64_t* tet0;
   const int32_t* ntet;
   const int32_t* prob;
@@ -187,18 +207,18 @@ struct BlockTable {
   int coupled;  // nonzero: the problems are the parts of one sharded problem; every problem's
                 // scalars are the sums over all blocks (the all-reduce of a sharded CG)
 };
-constexpr int DOT_THREADS = 128;
+constexpr int DOT_TETS = 128;  // tetrahedra of a reduction block
+constexpr int DOT_THREADS = 2 * DOT_TETS;
 
-// Layout conversion over (tet, c in [0, cnt), node):
-//   internal [tile][ncomp_in][np][32] at component c_in0 + c  <->  external [tet][ncomp_ext][np] at c_ext0 + c.
-// to_internal multiplies by scale (and by per_tet[e] if non-null); padding tets get 0.
+// Conversion between boundary arrays (nodal values in double) and a field vector: field f of
+// tetrahedron e has component c's nodes at x_f[e * stride + c * Np].  to_internal multiplies by
+// per_tet[e] if non-null, reads a null x1 as zeros and gives padding 0.
 template <typename R>
-void launch_to_internal(const double* ext, int ncomp_ext, int c_ext0, R* in, int ncomp_in, int c_in0, int cnt,
-                        const int32_t* ext_of_int, int64_t nti, int np, double scale, const double* per_tet,
-                        cudaStream_t s);
+void launch_to_internal(int q, const double* x0, const double* x1, int64_t stride, R* in, const int32_t* ext_of_int,
+                        int64_t nti, const double* per_tet, cudaStream_t s);
 template <typename R>
-void launch_to_external(const R* in, int ncomp_in, int c_in0, double* ext, int ncomp_ext, int c_ext0, int cnt,
-                        const int32_t* ext_of_int, int64_t nti, int np, cudaStream_t s);
+void launch_to_external(int q, const R* in, double* x0, double* x1, int64_t stride, const int32_t* ext_of_int,
+                        int64_t nti, cudaStream_t s);
 // o1 = o2 = o3 = a x + b y (null outputs skipped, y may be null).
 template <typename R>
 void launch_lincomb3(R* o1, R* o2, R* o3, double a, const R* x, double b, const R* y, int64_t n, cudaStream_t s);
@@ -229,11 +249,11 @@ template <typename R>
 void launch_halo(R* v, const int64_t* dst, const int64_t* src, int64_t n, int np, cudaStream_t s);
 // wdot = 0 for the listed internal tetrahedra (ghosts do not count in the inner products).
 void launch_zero_wdot(double* wdot, const int64_t* tets, int64_t n, cudaStream_t s);
-// gvol item `item` of a problem's internal tetrahedra [0, nti) = val[e] * scale[e], e = e_of_i[i]
-// (device arrays in the problem's external order; padding gets 0).
+// sigma/eps of a problem's internal tetrahedra [0, nti) = val[e] * scale[e], e = e_of_i[i] (device
+// arrays in the problem's external order; padding gets 0); geo: the problem's first half tile.
 template <typename R>
-void launch_set_gvol_item(R* gvol, int item, const double* val, const double* scale, const int32_t* e_of_i,
-                          int64_t nti, cudaStream_t s);
+void launch_set_sigma(R* geo, const double* val, const double* scale, const int32_t* e_of_i, int64_t nti,
+                      cudaStream_t s);
 // D = R + beta_p D and Uw = D on the tiles of active problems.
 template <typename R>
 void launch_cg_direction(R* D, R* Uw, const R* Rv, const Scalars* sc, const int32_t* tprob, const int32_t* pactive,
@@ -247,6 +267,7 @@ void launch_cg_direction(R* D, R* Uw, const R* Rv, const Scalars* sc, const int3
 // Problems with pactive[p] == 0 are left alone for which 1 and 2.
 void launch_finalize(const double* partials, const BlockTable& bt, Scalars* sc, int32_t* pactive, const int32_t* used,
                      int which, double tol, cudaStream_t s);
+
 void upload_dot_mass(int q, const double* M);
 
 // Gauss-Legendre rule on [0, 1] (refelem.cpp).

@@ -4,9 +4,9 @@
 // and the lift LIFT . f of the face fluxes.  FP32 sweeps only; included by
 // dg_stage.cuh inside its anonymous namespace, once per order.
 //
-// Mapping.  A CTA of 128 threads covers 64 tetrahedra (two 32-tetrahedron
-// tiles); thread t is row t of every MMA and lane t of tensor memory (TMEM), and,
-// as in dg_stage_kernel, threads 2k and 2k + 1 hold the electric and the magnetic
+// Mapping.  A CTA of 128 threads covers 64 tetrahedra (four half tiles, one per
+// warp); thread t is row t of every MMA and lane t of tensor memory (TMEM), and,
+// as in dg_stage_kernel, lanes 2k and 2k + 1 hold the electric and the magnetic
 // field of one tetrahedron (each computes the other field's Phi).  Per row:
 //
 //   volume:  d_{c'}[(b, i)] = sum_j F_{c'}[j] D_b[i][j]      (3 MMAs chains, K = Np, N = 3 Np)
@@ -157,64 +157,51 @@ template <int MINB>
 __global__ void __launch_bounds__(TC_THREADS, MINB) dg_stage_tc(const StageArgs<float> a) {
   using R = float;
   constexpr int NP = NPQ, NFP = NFPQ;
-  constexpr int VS = 6 * NP * TILE;
   constexpr FaceTab FM = make_fmask(CMCG_Q);
   constexpr uint32_t IDV = tc_idesc(128, TC_NV), IDL = tc_idesc(128, TC_NL);
   grid_dep_launch();
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const int64_t gthr = (int64_t)blockIdx.x * TC_THREADS + tid;
-  const int64_t gt = gthr >> 1;
-  const int half = int(gthr & 1);  // 0: owns E, computes Phi_H;  1: owns H, computes Phi_E
-  const int64_t tile = gt >> 5;
-  const int lane = int(gt & 31);
-  const bool in_range = gt < a.nti;  // warp-uniform (nti is a multiple of 32)
+  const int tid = threadIdx.x, warp = tid >> 5, l = tid & 31, half = l & 1;
+  const int64_t ht = int64_t(blockIdx.x) * (TC_THREADS / 32) + warp;
+  const bool in_range = ht * HTILE < a.nti;  // warp-uniform
 
   __shared__ __align__(8) uint64_t bars[3];  // [0]: reference matrices loaded, [1 + b]: MMAs of buffer b
   __shared__ uint32_t tmem_base;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   unsigned char* sB = smem_raw;                                            // TC_B_BYTES
   R* tr = reinterpret_cast<R*>(smem_raw + TC_B_BYTES) + tid;               // trace / flux slots
-  R* bs = tr + TRACE_SLOTS * TC_THREADS;                                   // base rows
-  R* js = bs + 3 * NP * TC_THREADS;  // source rows (single-frequency source stages): J_re (half 1), J_im (half 0)
-  const bool jpre = a.jre && a.nharm <= 0;
+  R* bs = tr + 4 * NFP * 3 * TC_THREADS;                                   // base rows
+  R* js = bs + 3 * NP * TC_THREADS;  // source rows (single-frequency source stages)
+  const bool jpre = a.j && a.nharm <= 0;
 
   int prob = 0;
   StageCoef<R> cf;
   cf.active = 0;
   if (in_range) {
-    prob = a.tprob ? a.tprob[tile] : 0;
+    prob = a.tprob ? a.tprob[ht >> 1] : 0;
     cf = a.coef[prob];
   }
   bool live = in_range && cf.active;
   if (!__syncthreads_or(live)) return;  // CTA-uniform
-  const int cOwn = half ? 3 : 0, cOut = half ? 0 : 3;
-  const R sH = a.sH;
-  const R sIn = half ? sH : R(1);
-  const R sOut = half ? R(1) : sH;
-  const R pec = half ? R(0) : R(-2);
-  R G[9], sv = 0;
-  int32_t code[4] = {NBR_PEC, NBR_PEC, NBR_PEC, NBR_PEC};
-  R fn[4][3], fk1[4], fk2[4];
+  // A warp without a half tile takes half tile 0's geometry and neighbours, and stores nothing.
+  const int64_t hr = in_range ? ht : 0;
+  R G[9];
 #pragma unroll
-  for (int m = 0; m < 9; ++m) G[m] = 0;
+  for (int m = 0; m < 9; ++m) G[m] = a.geo[hr * GEO32 + m * 16 + (l >> 1)];
+  const R sv = a.geo[hr * GEO32 + GEO_S32 * 16 + l] * a.sH;
+  struct Face {
+    R n[3], k1, k2;
+    Neighbour<R> nb;
+  } F[4];
 #pragma unroll
-  for (int f = 0; f < 4; ++f) fn[f][0] = fn[f][1] = fn[f][2] = fk1[f] = fk2[f] = 0;
-  if (live) {
-    const R* gv = a.gvol + tile * GV * TILE + lane;
+  for (int f = 0; f < 4; ++f) {
 #pragma unroll
-    for (int m = 0; m < 9; ++m) G[m] = gv[m * TILE];
-    sv = half ? -gv[9 * TILE] : gv[10 * TILE] * sOut;
-#pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      code[f] = a.nbr[(tile * 4 + f) * TILE + lane];
-      const R* gf = a.gface + (tile * 4 + f) * GF * TILE + lane;
-      fn[f][0] = gf[0];
-      fn[f][1] = gf[TILE];
-      fn[f][2] = gf[2 * TILE];
-      fk1[f] = gf[(3 + 2 * half) * TILE] * sOut;
-      fk2[f] = gf[(4 + 2 * half) * TILE] * sOut;
-    }
+    for (int k = 0; k < 3; ++k) F[f].n[k] = a.geo[hr * GEO32 + (9 + 3 * f + k) * 16 + (l >> 1)];
+    const R* gp = a.geo + hr * GEO32 + GEO_S32 * 16 + (1 + 2 * f) * 32 + l;
+    F[f].k1 = gp[0] * a.sH;
+    F[f].k2 = gp[32];
+    F[f].nb = find_neighbour(a, hr, l, f);
   }
+  const R sigma = a.sigma ? a.geo[hr * GEO32 + (GEO_S32 * 16 + GEO_SIGMA * 32) + l] : R(0);
   // The reference matrices (written only at handle creation) are copied before the grid
   // dependency: one bulk copy, completion counted in bytes on barB.
   const uint32_t barB = smem_addr(&bars[0]);
@@ -246,41 +233,28 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) dg_stage_tc(const StageArgs<
 
   // Own field, neighbour traces, base rows and (single-frequency source stages) source rows.
   R v[3][NP];
-  const int64_t off = tile * VS + cOut * NP * TILE + lane;
+  const int64_t own = hr * HS + l;  // the thread's field; its output is the partner's, own ^ 1
 #pragma unroll
   for (int c = 0; c < 3; ++c)
 #pragma unroll
-    for (int n = 0; n < NP; ++n) v[c][n] = R(0);
-  if (live) {
-    const R* vin = a.vin + tile * VS + cOwn * NP * TILE + lane;
+    for (int n = 0; n < NP; ++n) v[c][n] = a.vin[own + (c * NP + n) * 32];
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
+  for (int f = 0; f < 4; ++f) {
+    const R* nb = a.vin + F[f].nb.at;
 #pragma unroll
-      for (int n = 0; n < NP; ++n) v[c][n] = sIn * vin[(c * NP + n) * TILE];
+    for (int jf = 0; jf < NFP; ++jf) {
+      const R* p = nb + (unsigned(F[f].nb.nodes >> (5 * jf)) & 31u) * 32u;
 #pragma unroll
-    for (int f = 0; f < 4; ++f) {
-      if (code[f] >= 0) {
-        const int64_t k = int64_t(code[f] >> 5);
-        const R* nb = a.vin + (k >> 5) * VS + cOwn * NP * TILE + (k & 31);
-        const int tab = (((code[f] >> 3) & 3) * 6 + (code[f] & 7)) * NFP;
-#pragma unroll
-        for (int jf = 0; jf < NFP; ++jf) {
-          const int nn = cNB[tab + jf];
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-            cp_async_4(tr + ((f * NFP + jf) * 3 + c) * TC_THREADS, nb + (c * NP + nn) * TILE);
-        }
-      }
+      for (int c = 0; c < 3; ++c) cp_async_4(tr + ((f * NFP + jf) * 3 + c) * TC_THREADS, p + c * NP * 32);
     }
-    if (a.out) {
+  }
+  if (a.out) {
 #pragma unroll
-      for (int k = 0; k < 3 * NP; ++k) cp_async_4(bs + k * TC_THREADS, a.base + off + k * TILE);
-    }
-    if (jpre) {
-      const R* src = (half ? a.jre : a.jim) + tile * (3 * NP * TILE) + lane;
+    for (int k = 0; k < 3 * NP; ++k) cp_async_4(bs + k * TC_THREADS, a.base + (own ^ 1) + k * 32);
+  }
+  if (jpre) {
 #pragma unroll
-      for (int k = 0; k < 3 * NP; ++k) cp_async_4(js + k * TC_THREADS, src + k * TILE);
-    }
+    for (int k = 0; k < 3 * NP; ++k) cp_async_4(js + k * TC_THREADS, a.j + own + k * 32);
   }
   cp_async_commit();
 
@@ -417,26 +391,17 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) dg_stage_tc(const StageArgs<
   }
 
   // Face fluxes (CUDA cores, overlapping the volume MMAs), stored over the trace slots.
-  cp_async_wait_all();
+  cp_async_wait<0>();
 #pragma unroll
   for (int f = 0; f < 4; ++f) {
-    const R n0 = fn[f][0], n1 = fn[f][1], n2 = fn[f][2];
-    const R k2 = fk2[f];
-    const R m0 = fk1[f] * n0, m1 = fk1[f] * n1, m2 = fk1[f] * n2;  // k1 n, once per face
-    const bool interior = code[f] >= 0;
-    const R bscale = code[f] == NBR_PEC ? pec : R(-1);
+    const R n0 = F[f].n[0], n1 = F[f].n[1], n2 = F[f].n[2], k2 = F[f].k2;
+    const R m0 = F[f].k1 * n0, m1 = F[f].k1 * n1, m2 = F[f].k1 * n2;  // k1 n, once per face
 #pragma unroll
     for (int jf = 0; jf < NFP; ++jf) {
-      const int own = FM.v[f][jf];
+      const int own_node = FM.v[f][jf];
       R X[3], Y[3];
-      // both jumps formed and one selected: one code path per face node (the trace slots of a
-      // boundary face hold stale values, which the selection discards)
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const R xi = sIn * tr[((f * NFP + jf) * 3 + c) * TC_THREADS] - v[c][own];
-        const R xb = bscale * v[c][own];
-        X[c] = interior ? xi : xb;
-      }
+      for (int c = 0; c < 3; ++c) X[c] = fmaf(F[f].nb.c, tr[((f * NFP + jf) * 3 + c) * TC_THREADS], -v[c][own_node]);
 #pragma unroll
       for (int c = 0; c < 3; ++c) Y[c] = __shfl_xor_sync(0xffffffffu, X[c], 1);
       const R nY = n0 * Y[0] + n1 * Y[1] + n2 * Y[2];
@@ -497,50 +462,29 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) dg_stage_tc(const StageArgs<
   }
   if (!live) return;
 
-  if (half && a.sigma) {  // conductivity: Phi_E -= (sigma / eps) E (E is not flipped by Sigma)
-    const R so = a.gvol[(tile * GV + 11) * TILE + lane];
-    const R* ev = a.vin + tile * VS + lane;
+  R jv[3][NP];
+  if (jpre) {
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
-      for (int n = 0; n < NP; ++n) phi[c][n] -= so * ev[(c * NP + n) * TILE];
+      for (int n = 0; n < NP; ++n) jv[c][n] = js[(c * NP + n) * TC_THREADS];
   }
-  if (half && jpre) {  // source on the E rows: J_re in this thread's slots, J_im in the partner's
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int n = 0; n < NP; ++n) {
-        const int k = (c * NP + n) * TC_THREADS;
-        phi[c][n] += cf.s_cos * js[k] - cf.s_sin * js[k - 1];
-      }
-  } else if (half && a.jre) {
-    add_source<R, NP>(phi, a, cf, tile, lane, 0);
-  }
-  if (a.bre) {  // impedance-face data on this thread's output rows (source sweeps only)
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int n = 0; n < NP; ++n) {
-        const int64_t o = off + (c * NP + n) * TILE;
-        phi[c][n] += cf.s_cos * a.bre[o] - cf.s_sin * a.bim[o];
-      }
-  }
-  if (a.fre) accumulate_filter<R, NP>(a, cf, phi, off, 0);  // forward sweeps with the filter only
+  add_data<R, NP>(phi, jv, a, cf, own, 0, half, sigma);
+  if (a.fre) accumulate_filter<R, NP>(a, cf, phi, own ^ 1, 0);  // forward sweeps with the filter only
   if (a.out) {
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
-      for (int n = 0; n < NP; ++n) {
-        const int64_t o = off + (c * NP + n) * TILE;
-        a.out[o] = bs[(c * NP + n) * TC_THREADS] + cf.c_out * phi[c][n];
-      }
+      for (int n = 0; n < NP; ++n)
+        a.out[(own ^ 1) + (c * NP + n) * 32] = bs[(c * NP + n) * TC_THREADS] + cf.c_out * phi[c][n];
   }
 }
 
 // Dynamic shared memory of dg_stage_tc: reference matrices, trace slots, base rows,
-// and the prefetched source rows of single-frequency source stages (src = true).
+// and the prefetched source rows of single-frequency source stages (src = true; J_re in the even
+// threads' slots, J_im in the odd ones').
 constexpr size_t tc_smem(bool src) {
-  return size_t(TC_B_BYTES) + size_t(TRACE_SLOTS + (src ? 6 : 3) * NPQ) * TC_THREADS * sizeof(float);
+  return size_t(TC_B_BYTES) + size_t(4 * NFPQ * 3 + (src ? 6 : 3) * NPQ) * TC_THREADS * sizeof(float);
 }
 // Resident CTAs per SM that the TMEM columns allow (512 per SM).
 constexpr int TC_MINB = 2;

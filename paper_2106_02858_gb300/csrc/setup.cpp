@@ -5,13 +5,13 @@
 // shape class (identical edge vectors up to 1e-9 relative, e.g. the six Kuhn
 // tetrahedra of a Cartesian mesh), each group is sorted by centroid (z, then y,
 // then x on a grid of a quarter of the smallest edge), and each group is padded
-// to a multiple of 32.  A tile of 32 consecutive internal tetrahedra is one warp
-// of the stage kernel; every per-tetrahedron quantity is stored [tile][item][lane]
-// so that a warp's loads are contiguous, and within a group neighbouring
-// tetrahedra across a given face sit in neighbouring lanes.  Meshes with more
-// than 64 shape classes form a single group sorted by centroid.  Padding
-// tetrahedra have zero geometry, PEC faces and zero weights, so their fields
-// stay zero.
+// to a multiple of 32; the half tiles are then interleaved over the groups.  A
+// half tile (16 tetrahedra) is one warp of the stage kernel; every quantity is
+// stored [half tile][item][place] so that a warp's loads are contiguous, and
+// within a tile the neighbours across a given face sit in neighbouring places.
+// Meshes with more than 64 shape classes form a single group sorted by
+// centroid.  Padding tetrahedra have zero geometry, PEC faces and zero weights,
+// so their fields stay zero.
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -19,7 +19,7 @@
 #include <tuple>
 #include <unordered_map>
 
-#include "common.h"
+#include "bernstein.h"
 
 namespace cmcg {
 namespace {
@@ -234,13 +234,31 @@ int validate_and_layout(const cmcg_mesh* mesh, const double* eps, const double* 
     if (xa != xb) return xa < xb;
     return a < b;
   });
+  // Half tiles of the groups one after another (each group padded to whole tiles), then all of them
+  // in the order of their relative position in their group: half tile h of every group of a Cartesian
+  // mesh holds the same 16 cubes, so the tetrahedra of a cube, which share faces, are worked on by
+  // neighbouring warps and their traces are read while they are in L1.
+  std::vector<int32_t> grouped;
+  grouped.reserve(nt + 32 * ngroups);
+  std::vector<double> pos;  // of each half tile in its group
+  for (int64_t i = 0; i < nt;) {
+    int64_t e = i;
+    while (e < nt && cls[order[e]] == cls[order[i]]) grouped.push_back((int32_t)order[e++]);
+    while (grouped.size() % TILE) grouped.push_back(-1);
+    const size_t n = grouped.size() / HTILE - pos.size();
+    for (size_t h = 0; h < n; ++h) pos.push_back((double(h) + 0.5) / double(n));
+    i = e;
+  }
+  std::vector<int32_t> place(pos.size());
+  for (size_t h = 0; h < place.size(); ++h) place[h] = int32_t(h);
+  std::stable_sort(place.begin(), place.end(), [&](int32_t a, int32_t b) { return pos[a] < pos[b]; });
   std::vector<int32_t> ext_of_int;
-  ext_of_int.reserve(nt + 32 * ngroups);
-  for (int64_t i = 0; i < nt; ++i) {
-    ext_of_int.push_back((int32_t)order[i]);
-    bool end_group = (i + 1 == nt) || cls[order[i + 1]] != cls[order[i]];
-    if (end_group)
-      while (ext_of_int.size() % TILE) ext_of_int.push_back(-1);
+  ext_of_int.reserve(grouped.size());
+  out->half_at.assign(place.size(), 0);
+  for (size_t h = 0; h < place.size(); ++h) {
+    out->half_at[place[h]] = int32_t(h);
+    ext_of_int.insert(ext_of_int.end(), grouped.begin() + int64_t(place[h]) * HTILE,
+                      grouped.begin() + (int64_t(place[h]) + 1) * HTILE);
   }
   const int64_t nti = (int64_t)ext_of_int.size();
   const int64_t ntiles = nti / TILE;
@@ -252,25 +270,50 @@ int validate_and_layout(const cmcg_mesh* mesh, const double* eps, const double* 
   out->ngroups = ngroups;
   out->nti = nti;
   out->ntiles = ntiles;
-  out->gvol.assign(ntiles * GV * TILE, 0.0);
-  out->gface.assign(ntiles * 4 * GF * TILE, 0.0);
-  out->nbr.assign(ntiles * 4 * TILE, NBR_PEC);
+  const bool fp32 = opt->precision == CMCG_FP32;
+  const int gs = fp32 ? GEO_S32 : GEO_S64, gsize = fp32 ? GEO32 : GEO64;
+  out->geo.assign(ntiles * 2 * gsize, 0.0);
+  out->nbr.resize(ntiles * 4 * TILE);
   out->wdot.assign(ntiles * 2 * TILE, 0.0);
+  out->imp.clear();
   const bool centred = opt->flux == CMCG_FLUX_CENTRED;
   for (int64_t i = 0; i < nti; ++i) {
     const int64_t e = ext_of_int[i];
-    if (e < 0) continue;
-    const int64_t tile = i / TILE, lane = i % TILE;
-    auto gv = [&](int item) -> double& { return out->gvol[(tile * GV + item) * TILE + lane]; };
-    for (int m = 0; m < 9; ++m) gv(m) = G[9 * e + m];
-    gv(9) = 1.0 / eps[e];
-    gv(10) = 1.0 / mu[e];
-    out->wdot[(tile * 2 + 0) * TILE + lane] = absdet[e] * eps[e];
-    out->wdot[(tile * 2 + 1) * TILE + lane] = absdet[e] * mu[e];
+    const int64_t ht = i / HTILE, l = i % HTILE;
+    auto code_at = [&](int f) -> int32_t& { return out->nbr[(ht * 4 + f) * HTILE + l]; };
+    if (e < 0) {
+      for (int f = 0; f < 4; ++f) code_at(f) = (int32_t(i) << 5) | (f << 3) | PERM_PEC;
+      continue;
+    }
+    auto shared = [&](int item) -> double& { return out->geo[ht * gsize + item * HTILE + l]; };
+    auto thread = [&](int item, int half) -> double& {
+      return out->geo[ht * gsize + gs * HTILE + item * 2 * HTILE + 2 * l + half];
+    };
+    for (int m = 0; m < 9; ++m) shared(m) = G[9 * e + m];
+    thread(0, 0) = 1.0 / mu[e];
+    thread(0, 1) = -1.0 / eps[e];
+    out->wdot[2 * i + 0] = absdet[e] * eps[e];
+    out->wdot[2 * i + 1] = absdet[e] * mu[e];
     const double Zm = std::sqrt(mu[e] / eps[e]), Ym = 1.0 / Zm;
     for (int f = 0; f < 4; ++f) {
-      auto gf = [&](int item) -> double& { return out->gface[((tile * 4 + f) * GF + item) * TILE + lane]; };
-      for (int a = 0; a < 3; ++a) gf(a) = nrm[12 * e + 3 * f + a];
+      const double* n = &nrm[12 * e + 3 * f];
+      if (fp32) {
+        for (int a = 0; a < 3; ++a) shared(9 + 3 * f + a) = n[a];
+      } else {
+        const double* xa = Xv + 3 * (int64_t)T[4 * e + FACE_VERTS[f][0]];
+        const double* xb = Xv + 3 * (int64_t)T[4 * e + FACE_VERTS[f][1]];
+        double t1[3], len = 0;
+        for (int a = 0; a < 3; ++a) {
+          t1[a] = xb[a] - xa[a];
+          len += t1[a] * t1[a];
+        }
+        for (int a = 0; a < 3; ++a) {
+          t1[a] /= std::sqrt(len);
+          shared(9 + 6 * f + a) = t1[a];
+        }
+        for (int a = 0; a < 3; ++a)
+          shared(9 + 6 * f + 3 + a) = n[(a + 1) % 3] * t1[(a + 2) % 3] - n[(a + 2) % 3] * t1[(a + 1) % 3];
+      }
       const double fscale = area[4 * e + f] / rm.face_ref_area[f] / absdet[e];
       double Zp = Zm, Yp = Ym;
       int32_t code;
@@ -294,18 +337,31 @@ int validate_and_layout(const cmcg_mesh* mesh, const double* eps, const double* 
         if (p < 0) return fail(why, "face vertices do not match", CMCG_ERR_NONCONFORMING_MESH);
         code = (int32_t(int_of_ext[en]) << 5) | (fn << 3) | p;
       } else {
-        code = mesh->face_tags[4 * e + f] == CMCG_TAG_PEC ? NBR_PEC : NBR_IMP;
+        const bool pec = mesh->face_tags[4 * e + f] == CMCG_TAG_PEC;
+        code = (int32_t(i) << 5) | (f << 3) | (pec ? PERM_PEC : PERM_IMP);
       }
-      out->nbr[(tile * 4 + f) * TILE + lane] = code;
+      code_at(f) = code;
       // E-rows flux  fE = aE (dE - n (n.dE)) - bE n x dH,  H-rows flux  fH = bH n x dE + aH (dH - n (n.dH))
       // with aE = fscale / (eps (Z- + Z+)), bE = Z+ aE, aH = fscale / (mu (Y- + Y+)), bH = Y+ aH.
-      // Stored per half of the thread pair: (k1, k2) = (bH, aH) for the thread that owns E and
-      // computes Phi_H, (-bE, aE) for the thread that owns H and computes Phi_E.
+      // Per thread: k1 of n x (own field's jump) and k2 of the partner's, (bH, aH) for the thread that
+      // owns E and computes Phi_H, (-bE, aE) for the one that owns H.  In FP64 the lift is that of
+      // BernTab, without the reference face's area, and k2 is given as its ratio to k1.
       const double aE = fscale / eps[e] / (Zm + Zp), aH = fscale / mu[e] / (Ym + Yp);
-      gf(3) = Yp * aH;
-      gf(4) = centred ? 0.0 : aH;
-      gf(5) = -Zp * aE;
-      gf(6) = centred ? 0.0 : aE;
+      const double r = fp32 ? 1.0 : 2.0 * rm.face_ref_area[f];
+      thread(1 + 2 * f, 0) = r * (Yp * aH);
+      thread(1 + 2 * f, 1) = r * (-Zp * aE);
+      thread(2 + 2 * f, 0) = centred ? 0.0 : fp32 ? aH : Zp;
+      thread(2 + 2 * f, 1) = centred ? 0.0 : fp32 ? aE : -Yp;
+      if (nkf < 0 && mesh->face_tags[4 * e + f] == CMCG_TAG_IMPEDANCE) {
+        ImpFace F;
+        F.it = i;
+        F.ext = int32_t(e);
+        F.f = f;
+        for (int a = 0; a < 3; ++a) F.n[a] = n[a];
+        F.aE = centred ? 0.0 : aE;
+        F.bH = Yp * aH;
+        out->imp.push_back(F);
+      }
     }
   }
   out->ext_of_int = std::move(ext_of_int);

@@ -1,66 +1,80 @@
 // Vector kernels of the CMCG outer loop (Section 2.2, Algorithm cmcg):
-// layout conversion between the boundary layout [tet][comp][node] (double) and
-// the device layout [tile][comp][node][lane], fused CG updates, and the
+// conversion between the boundary layout [tet][comp][node] (nodal values, double) and
+// the handle's fields (field_at; nodal values in FP32, Bernstein coefficients in FP64),
+// fused CG updates, and the
 // (eps, mu)-weighted inner product (Eq. innerproduct)
 //     (X, Y) = sum_K |det A_K| sum_c w_c sum_ij X_c[i] Mref[i][j] Y_c[j],
 // w_c = eps_K on E rows, mu_K on H rows, accumulated in FP64 whatever the
 // storage precision.  Reductions are deterministic: one partial per block
 // (warp shuffles, then shared memory in a fixed order) and one finalising
 // block that sums the partials in a fixed order.
-#include "common.h"
+#include "bernstein.h"
 
 namespace cmcg {
 namespace {
 
-
-__constant__ double cM1[4 * 4];
-__constant__ double cM2[10 * 10];
-__constant__ double cM3[20 * 20];
-
-template <int Q>
-__device__ __forceinline__ double cM(int idx) {
-  if constexpr (Q == 1) return cM1[idx];
-  else if constexpr (Q == 2) return cM2[idx];
-  else return cM3[idx];
-}
-
-template <typename R>
-__global__ void to_internal_kernel(const double* __restrict__ ext, int ncomp_ext, int c_ext0, R* __restrict__ in,
-                                   int ncomp_in, int c_in0, int cnt, const int32_t* __restrict__ e_of_i, int64_t nti,
-                                   int np, double scale, const double* __restrict__ per_tet) {
-  const int64_t total = nti * cnt * np;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int lane = int(idx % TILE);
-    const int64_t r = idx / TILE;
-    const int n = int(r % np);
-    const int c = int((r / np) % cnt);
-    const int64_t tile = r / ((int64_t)np * cnt);
-    const int32_t e = e_of_i[tile * TILE + lane];
-    R v = R(0);
-    if (e >= 0) {
-      double x = ext[((int64_t)e * ncomp_ext + c_ext0 + c) * np + n] * scale;
-      if (per_tet) x *= per_tet[e];
-      v = R(x);
+// One warp converts one component of a half tile: lane 2t + f takes field f of tetrahedron t, its
+// nodes being contiguous in the boundary arrays.  x0, x1: the arrays of the two fields, at
+// [tet * stride + c * Np] (x1 null: zeros).
+template <int Q, typename R>
+__global__ void __launch_bounds__(128) to_internal_kernel(const double* x0, const double* x1, int64_t stride, R* in,
+                                                          const int32_t* e_of_i, int64_t nti, const double* per_tet) {
+  constexpr int NP = np_of(Q);
+  constexpr BasisRows<Q> T = make_to_bern<Q>();
+  const int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  const int64_t ht = w / 3;
+  const int c = int(w % 3), l = threadIdx.x & 31;
+  if (ht * HTILE >= nti) return;
+  const int32_t e = e_of_i[ht * HTILE + (l >> 1)];
+  const double* x = (l & 1) ? x1 : x0;
+  double u[NP];
+#pragma unroll
+  for (int n = 0; n < NP; ++n) u[n] = 0;
+  if (e >= 0 && x) {
+    x += e * stride + c * NP;
+    const double s = per_tet ? per_tet[e] : 1.0;
+#pragma unroll
+    for (int n = 0; n < NP; ++n) u[n] = x[n] * s;
+  }
+  R* o = in + ht * (96 * NP) + c * NP * 32 + l;
+#pragma unroll
+  for (int n = 0; n < NP; ++n) {
+    double v = u[n];
+    if constexpr (sizeof(R) == 8) {
+      v = T.r[n].w[0] * u[T.r[n].col[0]];
+#pragma unroll
+      for (int k = 1; k < 10; ++k)
+        if (k < T.r[n].n) v = fma(T.r[n].w[k], u[T.r[n].col[k]], v);
     }
-    in[((tile * ncomp_in + c_in0 + c) * np + n) * TILE + lane] = v;
+    o[n * 32] = R(v);
   }
 }
 
-template <typename R>
-__global__ void to_external_kernel(const R* __restrict__ in, int ncomp_in, int c_in0, double* __restrict__ ext,
-                                   int ncomp_ext, int c_ext0, int cnt, const int32_t* __restrict__ e_of_i, int64_t nti,
-                                   int np) {
-  const int64_t total = nti * cnt * np;
-  for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total;
-       idx += (int64_t)gridDim.x * blockDim.x) {
-    const int lane = int(idx % TILE);
-    const int64_t r = idx / TILE;
-    const int n = int(r % np);
-    const int c = int((r / np) % cnt);
-    const int64_t tile = r / ((int64_t)np * cnt);
-    const int32_t e = e_of_i[tile * TILE + lane];
-    if (e >= 0) ext[((int64_t)e * ncomp_ext + c_ext0 + c) * np + n] = double(in[((tile * ncomp_in + c_in0 + c) * np + n) * TILE + lane]);
+template <int Q, typename R>
+__global__ void __launch_bounds__(128) to_external_kernel(const R* in, double* x0, double* x1, int64_t stride,
+                                                          const int32_t* e_of_i, int64_t nti) {
+  constexpr int NP = np_of(Q);
+  constexpr BasisRows<Q> T = make_to_node<Q>();
+  const int64_t w = (int64_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+  const int64_t ht = w / 3;
+  const int c = int(w % 3), l = threadIdx.x & 31;
+  if (ht * HTILE >= nti) return;
+  const int32_t e = e_of_i[ht * HTILE + (l >> 1)];
+  double u[NP];
+#pragma unroll
+  for (int n = 0; n < NP; ++n) u[n] = double(in[ht * (96 * NP) + (c * NP + n) * 32 + l]);
+  if (e < 0) return;
+  double* x = ((l & 1) ? x1 : x0) + e * stride + c * NP;
+#pragma unroll
+  for (int n = 0; n < NP; ++n) {
+    double v = u[n];
+    if constexpr (sizeof(R) == 8) {
+      v = T.r[n].w[0] * u[T.r[n].col[0]];
+#pragma unroll
+      for (int k = 1; k < 10; ++k)
+        if (k < T.r[n].n) v = fma(T.r[n].w[k], u[T.r[n].col[k]], v);
+    }
+    x[n] = v;
   }
 }
 
@@ -92,88 +106,157 @@ __global__ void lincomb_kernel(R* o1, R* o2, R* o3, double a, const R* x, double
   }
 }
 
-__device__ __forceinline__ double block_sum(double v) {
-  __shared__ double sh[DOT_THREADS / 32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  __syncthreads();  // a previous call's reads of sh are done
-  if (l == 0) sh[w] = v;
-  __syncthreads();
+// The element inner product on nodal values (FP32 fields): s_c = sum_i x_i (sum_j M_ij y_j), FP64.
+__constant__ double cM1[4 * 4];
+__constant__ double cM2[10 * 10];
+__constant__ double cM3[20 * 20];
+
+template <int Q>
+__device__ __forceinline__ double cM(int idx) {
+  if constexpr (Q == 1) return cM1[idx];
+  else if constexpr (Q == 2) return cM2[idx];
+  else return cM3[idx];
+}
+template <int Q>
+__device__ __forceinline__ double nodal_dot(const double (&x)[np_of(Q)], const double (&y)[np_of(Q)]) {
+  constexpr int NP = np_of(Q);
   double s = 0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < DOT_THREADS / 32; ++i) s += sh[i];
+#pragma unroll
+  for (int i = 0; i < NP; ++i) {
+    double t = 0;
+#pragma unroll
+    for (int j = 0; j < NP; ++j) t = fma(cM<Q>(i * NP + j), y[j], t);
+    s = fma(x[i], t, s);
+  }
   return s;
 }
 
-// Per-tet weighted dot of X and Y (vectors in device layout).
-template <int Q, typename R>
-__device__ __forceinline__ double tet_dot(const R* X, const R* Y, int64_t tile, int lane, const double* wdot) {
+// The element inner product on Bernstein coefficients (FP64 fields) as a sum of squares (bernstein.h): x^T M y = s sum_g X_g Y_g over the
+// degree-q coefficients and their contractions to every lower degree.  At GB300's FP64 rate the
+// operations bound these kernels: 60 contractions per vector and 35 products per pair at P3 (20 and
+// 15 at P2) where the dense mass matrix takes 420 (110).
+template <int Q>
+struct MassTab {
+  int dn[Q + 1][np_of(Q)][4];  // [k][g][i]: index of g + e_i in degree Q - k + 1, |g| = Q - k
+  int w[Q + 1][np_of(Q)][4];   // g_i + 1
+};
+template <int Q>
+constexpr MassTab<Q> make_mass() {
+  MassTab<Q> t{};
+  for (int k = 1; k <= Q; ++k)
+    for (int m = 0; m < np_of(Q - k); ++m)
+      for (int i = 0; i < 4; ++i) {
+        Bary4 g = bary_of(Q - k, m);
+        g.b[i] += 1;
+        t.dn[k][m][i] = node_at(Q - k + 1, g);
+        t.w[k][m][i] = g.b[i];
+      }
+  return t;
+}
+constexpr double mass_scale(int q) { return q == 1 ? 1.0 / 120 : q == 2 ? 1.0 / 1260 : 1.0 / 10080; }
+
+// x becomes its contraction to degree Q - k (x k!: the contractions are kept unnormalised).
+template <int Q, int K>
+__device__ __forceinline__ void contract(double (&x)[np_of(Q)]) {
+  constexpr MassTab<Q> T = make_mass<Q>();
+  double r[np_of(Q - K)];
+#pragma unroll
+  for (int m = 0; m < np_of(Q - K); ++m) {
+    double v = T.w[K][m][0] == 1 ? x[T.dn[K][m][0]] : T.w[K][m][0] * x[T.dn[K][m][0]];
+#pragma unroll
+    for (int i = 1; i < 4; ++i) v = fma(double(T.w[K][m][i]), x[T.dn[K][m][i]], v);
+    r[m] = v;
+  }
+#pragma unroll
+  for (int m = 0; m < np_of(Q - K); ++m) x[m] = r[m];
+}
+// xx += sum_g (x_g / k!)^2 over this degree and all lower ones (XX), xy the same with x_g y_g (XY).
+template <int Q, int K, bool XX, bool XY>
+__device__ __forceinline__ void mass_levels(double (&x)[np_of(Q)], double (&y)[np_of(Q)], double& xx, double& xy) {
+  if constexpr (K > 0) {
+    contract<Q, K>(x);
+    if constexpr (XY) contract<Q, K>(y);
+  }
+  constexpr int f = K == 2 ? 2 : K == 3 ? 6 : 1;  // K!
+  double a = 0, b = 0;
+#pragma unroll
+  for (int m = 0; m < np_of(Q - K); ++m) {
+    if constexpr (XX) a = fma(x[m], x[m], a);
+    if constexpr (XY) b = fma(x[m], y[m], b);
+  }
+  if constexpr (XX) xx = fma(a, 1.0 / (f * f), xx);
+  if constexpr (XY) xy = fma(b, 1.0 / (f * f), xy);
+  if constexpr (K < Q) mass_levels<Q, K + 1, XX, XY>(x, y, xx, xy);
+}
+
+// Block b of the table covers its tetrahedra in order, two threads each: the thread's internal
+// tetrahedron, or -1 when past the block's range.
+__device__ __forceinline__ int64_t block_tet(const BlockTable& bt) {
+  const int b = blockIdx.x, k = threadIdx.x >> 1;
+  if (k >= bt.ntet[b]) return -1;
+  const int64_t t = bt.tet0[b] + k;
+  return int64_t(bt.half_at[t >> 4]) * HTILE + (t & 15);
+}
+
+// Sum over the block of the odd threads' values: a warp's shuffle tree over 32 consecutive
+// tetrahedra, then the four warps' sums in order (valid in thread 0).
+__device__ __forceinline__ double block_sum(double v) {
+  __shared__ double tet[DOT_TETS];
+  __shared__ double sh[DOT_TETS / 32];
+  __syncthreads();  // a previous call's reads are done
+  if (threadIdx.x & 1) tet[threadIdx.x >> 1] = v;
+  __syncthreads();
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  if (w < DOT_TETS / 32) {
+    double x = tet[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (l == 0) sh[w] = x;
+  }
+  __syncthreads();
+  double s = 0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < DOT_TETS / 32; ++i) s += sh[i];
+  return s;
+}
+
+// The tetrahedron's products xx = (x, x) and xy = (x, y), valid in the odd thread; `load(c, x, y)`
+// loads component c of the thread's field.  FP32 fields keep one chain over the six components: the
+// odd thread goes on from the even thread's sum over E.
+template <int Q, typename R, bool XX, bool XY, typename Load>
+__device__ __forceinline__ void tet_dots(bool live, double w, double& xx, double& xy, Load&& load) {
   constexpr int NP = np_of(Q);
-  const R* x = X + tile * (6 * NP * TILE) + lane;
-  const R* y = Y + tile * (6 * NP * TILE) + lane;
-  const double wE = wdot[(tile * 2 + 0) * TILE + lane], wH = wdot[(tile * 2 + 1) * TILE + lane];
-  double total = 0;
+  double px[3] = {0, 0, 0}, py[3] = {0, 0, 0};
+  if (live)
 #pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    double yv[NP];
-#pragma unroll
-    for (int j = 0; j < NP; ++j) yv[j] = double(y[(c * NP + j) * TILE]);
+    for (int c = 0; c < 3; ++c) {
+      double x[NP], y[NP];
+      load(c, x, y);
+      if constexpr (sizeof(R) == 8) {
+        mass_levels<Q, 0, XX, XY>(x, y, px[c], py[c]);
+      } else {
+        if constexpr (XY) py[c] = nodal_dot<Q>(x, y);
+        if constexpr (XX) px[c] = nodal_dot<Q>(x, x);
+      }
+    }
+  if constexpr (sizeof(R) == 8) w *= mass_scale(Q);
+  auto chain = [&](const double (&p)[3]) {
     double s = 0;
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      double t = 0;
+    for (int c = 0; c < 3; ++c) s = fma(w, p[c], s);
+    const double e = __shfl_xor_sync(0xffffffffu, s, 1);
+    if (threadIdx.x & 1) {
+      s = e;
 #pragma unroll
-      for (int j = 0; j < NP; ++j) t = fma(cM<Q>(i * NP + j), yv[j], t);
-      s = fma(double(x[(c * NP + i) * TILE]), t, s);
+      for (int c = 0; c < 3; ++c) s = fma(w, p[c], s);
     }
-    total += (c < 3 ? wE : wH) * s;
-  }
-  return total;
+    return s;
+  };
+  if constexpr (XX) xx = chain(px);
+  if constexpr (XY) xy = chain(py);
 }
 
-// (X, Y) and (X, X) of one tetrahedron in one pass over X (each sum in the order of tet_dot).
-template <int Q, typename R>
-__device__ __forceinline__ void tet_dot2(const R* X, const R* Y, int64_t tile, int lane, const double* wdot,
-                                         double& xy, double& xx) {
-  constexpr int NP = np_of(Q);
-  const R* x = X + tile * (6 * NP * TILE) + lane;
-  const R* y = Y + tile * (6 * NP * TILE) + lane;
-  const double wE = wdot[(tile * 2 + 0) * TILE + lane], wH = wdot[(tile * 2 + 1) * TILE + lane];
-  xy = 0;
-  xx = 0;
-#pragma unroll
-  for (int c = 0; c < 6; ++c) {
-    double xv[NP], yv[NP];
-#pragma unroll
-    for (int j = 0; j < NP; ++j) {
-      xv[j] = double(x[(c * NP + j) * TILE]);
-      yv[j] = double(y[(c * NP + j) * TILE]);
-    }
-    double s = 0, s2 = 0;
-#pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      double t = 0, t2 = 0;
-#pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        t = fma(cM<Q>(i * NP + j), yv[j], t);
-        t2 = fma(cM<Q>(i * NP + j), xv[j], t2);
-      }
-      s = fma(xv[i], t, s);
-      s2 = fma(xv[i], t2, s2);
-    }
-    xy += (c < 3 ? wE : wH) * s;
-    xx += (c < 3 ? wE : wH) * s2;
-  }
-}
-
-// Block b of the table: its tets, or -1 when past the block's range.
-__device__ __forceinline__ int64_t block_tet(const BlockTable& bt) {
-  const int b = blockIdx.x;
-  return threadIdx.x < bt.ntet[b] ? bt.tet0[b] + threadIdx.x : -1;
-}
-
-// A = Uw - WT; partial (D, A).
+// A = Uw - WT; partials (D, A) and (D, D).
 template <int Q, typename R>
 __global__ void __launch_bounds__(DOT_THREADS) cg_after_adjoint_kernel(const R* Uw, const R* WT, R* A, const R* D,
                                                                       const double* wdot, double* partials,
@@ -181,16 +264,21 @@ __global__ void __launch_bounds__(DOT_THREADS) cg_after_adjoint_kernel(const R* 
   constexpr int NP = np_of(Q);
   const bool act = !pactive || pactive[bt.prob[blockIdx.x]];
   const int64_t t = block_tet(bt);
-  double acc = 0, dd = 0;
-  if (act && t >= 0) {
-    const int64_t tile = t >> 5;
-    const int lane = int(t & 31);
-    const int64_t base = tile * (6 * NP * TILE) + lane;
+  const bool live = act && t >= 0;
+  const int64_t o = live ? field_at(NP, t, threadIdx.x & 1, 0, 0) : 0;
+  double da = 0, dd = 0;
+  tet_dots<Q, R, true, true>(live, live ? wdot[2 * t + (threadIdx.x & 1)] : 0.0, dd, da,
+                       [&](int c, double (&x)[NP], double (&y)[NP]) {
 #pragma unroll
-    for (int k = 0; k < 6 * NP; ++k) A[base + k * TILE] = R(double(Uw[base + k * TILE]) - double(WT[base + k * TILE]));
-    tet_dot2<Q, R>(D, A, tile, lane, wdot, acc, dd);
-  }
-  const double s = block_sum(acc);
+                         for (int n = 0; n < NP; ++n) {
+                           const int64_t k = o + (c * NP + n) * 32;
+                           const R v = R(double(Uw[k]) - double(WT[k]));
+                           A[k] = v;
+                           y[n] = double(v);
+                           x[n] = double(D[k]);
+                         }
+                       });
+  const double s = block_sum(da);
   const double s2 = block_sum(dd);
   if (threadIdx.x == 0) {
     partials[blockIdx.x] = s;
@@ -207,70 +295,88 @@ __global__ void __launch_bounds__(DOT_THREADS) cg_update_kernel(R* U0, R* Rv, co
   const int p = bt.prob[blockIdx.x];
   const bool act = !pactive || pactive[p];
   const int64_t t = block_tet(bt);
-  double acc = 0;
-  if (act && t >= 0) {
-    const double alpha = sc[p].alpha;
-    const int64_t tile = t >> 5;
-    const int lane = int(t & 31);
-    const int64_t base = tile * (6 * NP * TILE) + lane;
+  const bool live = act && t >= 0;
+  const double alpha = act ? sc[p].alpha : 0.0;
+  const int64_t o = live ? field_at(NP, t, threadIdx.x & 1, 0, 0) : 0;
+  double rr = 0, unused = 0;
+  tet_dots<Q, R, true, false>(live, live ? wdot[2 * t + (threadIdx.x & 1)] : 0.0, rr, unused,
+                        [&](int c, double (&x)[NP], double (&y)[NP]) {
 #pragma unroll
-    for (int k = 0; k < 6 * NP; ++k) {
-      const int64_t o = base + k * TILE;
-      U0[o] = R(double(U0[o]) + alpha * double(D[o]));
-      Rv[o] = R(double(Rv[o]) - alpha * double(A[o]));
-    }
-    acc = tet_dot<Q, R>(Rv, Rv, tile, lane, wdot);
-  }
-  const double s = block_sum(acc);
+                          for (int n = 0; n < NP; ++n) {
+                            const int64_t k = o + (c * NP + n) * 32;
+                            U0[k] = R(double(U0[k]) + alpha * double(D[k]));
+                            const R r = R(double(Rv[k]) - alpha * double(A[k]));
+                            Rv[k] = r;
+                            x[n] = double(r);
+                          }
+                        });
+  const double s = block_sum(rr);
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
 template <int Q, typename R>
 __global__ void __launch_bounds__(DOT_THREADS) dot_kernel(const R* X, const R* Y, const double* wdot, double* partials,
                                                          const BlockTable bt) {
+  constexpr int NP = np_of(Q);
   const int64_t t = block_tet(bt);
-  const double acc = t >= 0 ? tet_dot<Q, R>(X, Y, t >> 5, int(t & 31), wdot) : 0.0;
+  const bool live = t >= 0;
+  const int64_t o = live ? field_at(NP, t, threadIdx.x & 1, 0, 0) : 0;
+  double acc = 0, unused = 0;
+  tet_dots<Q, R, false, true>(live, live ? wdot[2 * t + (threadIdx.x & 1)] : 0.0, unused, acc,
+                       [&](int c, double (&x)[NP], double (&y)[NP]) {
+#pragma unroll
+                         for (int n = 0; n < NP; ++n) {
+                           x[n] = double(X[o + (c * NP + n) * 32]);
+                           y[n] = double(Y[o + (c * NP + n) * 32]);
+                         }
+                       });
   const double s = block_sum(acc);
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 
+// Rows [tet][6][Np] into field vectors.
 template <typename R>
 __global__ void scatter_rows_kernel(R* dst_re, R* dst_im, const double* src_re, const double* src_im,
-                                    const int64_t* tet, int64_t count, int rows) {
-  const int64_t n = count * rows;
+                                    const int64_t* tet, int64_t count, int np) {
+  const int64_t rows = 6 * np, n = count * rows;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = i / rows, k = i % rows, t = tet[e];
-    const int64_t o = (t >> 5) * rows * TILE + k * TILE + (t & 31);
+    const int64_t e = i / rows;
+    const int k = int(i % rows);
+    const int64_t o = field_at(np, tet[e], k / (3 * np), k / np % 3, k % np);
     dst_re[o] = R(src_re[i]);
     dst_im[o] = R(src_im[i]);
   }
 }
 
 template <typename R>
-__global__ void halo_kernel(R* v, const int64_t* dst, const int64_t* src, int64_t n, int rows) {
-  const int64_t total = n * rows;
+__global__ void halo_kernel(R* v, const int64_t* dst, const int64_t* src, int64_t n, int np) {
+  const int64_t rows = 6 * np, total = n * rows;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t e = i / rows, k = i % rows, d = dst[e], s = src[e];
-    v[(d >> 5) * rows * TILE + k * TILE + (d & 31)] = v[(s >> 5) * rows * TILE + k * TILE + (s & 31)];
+    const int64_t e = i / rows;
+    const int k = int(i % rows), f = k & 1, m = k >> 1;  // the two fields of a coefficient are adjacent
+    v[field_at(np, dst[e], f, 0, m)] = v[field_at(np, src[e], f, 0, m)];
   }
 }
 
 __global__ void zero_wdot_kernel(double* wdot, const int64_t* tets, int64_t n) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     const int64_t t = tets[i];
-    wdot[((t >> 5) * 2 + 0) * TILE + (t & 31)] = 0.0;
-    wdot[((t >> 5) * 2 + 1) * TILE + (t & 31)] = 0.0;
+    wdot[2 * t] = 0.0;
+    wdot[2 * t + 1] = 0.0;
   }
 }
 
-// gvol item `item` of internal tetrahedra [0, nti) of one problem: val[e] * scale[e] for the
-// external tetrahedron e = e_of_i[i] (0 on padding).
+// sigma/eps of internal tetrahedra [0, nti) of one problem: val[e] * scale[e] for the external
+// tetrahedron e = e_of_i[i] (0 on padding).
 template <typename R>
-__global__ void set_gvol_item_kernel(R* gvol, int item, const double* val, const double* scale,
-                                     const int32_t* e_of_i, int64_t nti) {
+__global__ void set_sigma_kernel(R* geo, const double* val, const double* scale, const int32_t* e_of_i, int64_t nti) {
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nti; i += (int64_t)gridDim.x * blockDim.x) {
     const int32_t e = e_of_i[i];
-    gvol[((i >> 5) * GV + item) * TILE + (i & 31)] = e >= 0 ? R(val[e] * scale[e]) : R(0);
+    const R s = e >= 0 ? R(val[e] * scale[e]) : R(0);
+    constexpr int gs = sizeof(R) == 4 ? GEO_S32 : GEO_S64, size = sizeof(R) == 4 ? GEO32 : GEO64;
+    R* g = geo + (i >> 4) * size + gs * 16 + GEO_SIGMA * 32 + 2 * (i & 15);
+    g[0] = s;
+    g[1] = s;
   }
 }
 
@@ -373,6 +479,13 @@ int grid_for(int64_t n, int threads) {
 
 }  // namespace
 
+#define CMCG_BY_ORDER(q, KERNEL, blocks, threads, ...)                          \
+  do {                                                                          \
+    if ((q) == 1) KERNEL<1, R><<<blocks, threads, 0, s>>>(__VA_ARGS__);         \
+    else if ((q) == 2) KERNEL<2, R><<<blocks, threads, 0, s>>>(__VA_ARGS__);    \
+    else KERNEL<3, R><<<blocks, threads, 0, s>>>(__VA_ARGS__);                  \
+  } while (0)
+
 void upload_dot_mass(int q, const double* M) {
   const int np = np_of(q);
   if (q == 1) cudaMemcpyToSymbol(cM1, M, sizeof(double) * np * np);
@@ -381,18 +494,16 @@ void upload_dot_mass(int q, const double* M) {
 }
 
 template <typename R>
-void launch_to_internal(const double* ext, int ncomp_ext, int c_ext0, R* in, int ncomp_in, int c_in0, int cnt,
-                        const int32_t* e_of_i, int64_t nti, int np, double scale, const double* per_tet, cudaStream_t s) {
-  const int64_t n = nti * cnt * np;
-  to_internal_kernel<R><<<grid_for(n, 256), 256, 0, s>>>(ext, ncomp_ext, c_ext0, in, ncomp_in, c_in0, cnt, e_of_i, nti,
-                                                         np, scale, per_tet);
+void launch_to_internal(int q, const double* x0, const double* x1, int64_t stride, R* in, const int32_t* e_of_i,
+                        int64_t nti, const double* per_tet, cudaStream_t s) {
+  const unsigned blocks = unsigned((nti / HTILE * 3 + 3) / 4);  // four warps a block
+  CMCG_BY_ORDER(q, to_internal_kernel, blocks, 128, x0, x1, stride, in, e_of_i, nti, per_tet);
 }
 template <typename R>
-void launch_to_external(const R* in, int ncomp_in, int c_in0, double* ext, int ncomp_ext, int c_ext0, int cnt,
-                        const int32_t* e_of_i, int64_t nti, int np, cudaStream_t s) {
-  const int64_t n = nti * cnt * np;
-  to_external_kernel<R><<<grid_for(n, 256), 256, 0, s>>>(in, ncomp_in, c_in0, ext, ncomp_ext, c_ext0, cnt, e_of_i, nti,
-                                                         np);
+void launch_to_external(int q, const R* in, double* x0, double* x1, int64_t stride, const int32_t* e_of_i, int64_t nti,
+                        cudaStream_t s) {
+  const unsigned blocks = unsigned((nti / HTILE * 3 + 3) / 4);
+  CMCG_BY_ORDER(q, to_external_kernel, blocks, 128, in, x0, x1, stride, e_of_i, nti);
 }
 template <typename R>
 void launch_lincomb3_masked(R* o1, R* o2, R* o3, double a, const R* x, double b, const R* y, int64_t n, int np,
@@ -405,49 +516,42 @@ void launch_lincomb3(R* o1, R* o2, R* o3, double a, const R* x, double b, const 
   lincomb_kernel<R><<<grid_for(n, 256), 256, 0, s>>>(o1, o2, o3, a, x, b, y, n);
 }
 
-#define CMCG_DISPATCH_Q(q, KERNEL, ...)                                             \
-  do {                                                                              \
-    if ((q) == 1) KERNEL<1, R><<<bt.nblk, DOT_THREADS, 0, s>>>(__VA_ARGS__);        \
-    else if ((q) == 2) KERNEL<2, R><<<bt.nblk, DOT_THREADS, 0, s>>>(__VA_ARGS__);   \
-    else KERNEL<3, R><<<bt.nblk, DOT_THREADS, 0, s>>>(__VA_ARGS__);                 \
-  } while (0)
-
 template <typename R>
 void launch_cg_after_adjoint(int q, const R* Uw, const R* WT, R* A, const R* D, const double* wdot, double* partials,
                              const BlockTable& bt, const int32_t* pactive, cudaStream_t s) {
-  CMCG_DISPATCH_Q(q, cg_after_adjoint_kernel, Uw, WT, A, D, wdot, partials, bt, pactive);
+  CMCG_BY_ORDER(q, cg_after_adjoint_kernel, bt.nblk, DOT_THREADS, Uw, WT, A, D, wdot, partials, bt, pactive);
 }
 template <typename R>
 void launch_cg_update(int q, R* U0, R* Rv, const R* D, const R* A, const double* wdot, const Scalars* sc,
                       double* partials, const BlockTable& bt, const int32_t* pactive, cudaStream_t s) {
-  CMCG_DISPATCH_Q(q, cg_update_kernel, U0, Rv, D, A, wdot, sc, partials, bt, pactive);
+  CMCG_BY_ORDER(q, cg_update_kernel, bt.nblk, DOT_THREADS, U0, Rv, D, A, wdot, sc, partials, bt, pactive);
 }
 template <typename R>
 void launch_dot(int q, const R* X, const R* Y, const double* wdot, double* partials, const BlockTable& bt,
                 cudaStream_t s) {
-  CMCG_DISPATCH_Q(q, dot_kernel, X, Y, wdot, partials, bt);
+  CMCG_BY_ORDER(q, dot_kernel, bt.nblk, DOT_THREADS, X, Y, wdot, partials, bt);
 }
 template <typename R>
 void launch_scatter_rows(R* dst_re, R* dst_im, const double* src_re, const double* src_im, const int64_t* tet,
                          int64_t count, int np, cudaStream_t s) {
   if (count <= 0) return;
   scatter_rows_kernel<R><<<grid_for(count * 6 * np, 256), 256, 0, s>>>(dst_re, dst_im, src_re, src_im, tet, count,
-                                                                         6 * np);
+                                                                         np);
 }
 template <typename R>
 void launch_halo(R* v, const int64_t* dst, const int64_t* src, int64_t n, int np, cudaStream_t s) {
   if (n <= 0) return;
-  halo_kernel<R><<<grid_for(n * 6 * np, 256), 256, 0, s>>>(v, dst, src, n, 6 * np);
+  halo_kernel<R><<<grid_for(n * 6 * np, 256), 256, 0, s>>>(v, dst, src, n, np);
 }
 void launch_zero_wdot(double* wdot, const int64_t* tets, int64_t n, cudaStream_t s) {
   if (n <= 0) return;
   zero_wdot_kernel<<<grid_for(n, 256), 256, 0, s>>>(wdot, tets, n);
 }
 template <typename R>
-void launch_set_gvol_item(R* gvol, int item, const double* val, const double* scale, const int32_t* e_of_i,
-                          int64_t nti, cudaStream_t s) {
+void launch_set_sigma(R* geo, const double* val, const double* scale, const int32_t* e_of_i, int64_t nti,
+                      cudaStream_t s) {
   if (nti <= 0) return;
-  set_gvol_item_kernel<R><<<grid_for(nti, 256), 256, 0, s>>>(gvol, item, val, scale, e_of_i, nti);
+  set_sigma_kernel<R><<<grid_for(nti, 256), 256, 0, s>>>(geo, val, scale, e_of_i, nti);
 }
 template <typename R>
 void launch_cg_direction(R* D, R* Uw, const R* Rv, const Scalars* sc, const int32_t* tprob, const int32_t* pactive,
@@ -460,10 +564,9 @@ void launch_finalize(const double* partials, const BlockTable& bt, Scalars* sc, 
 }
 
 #define CMCG_INST(R)                                                                                                  \
-  template void launch_to_internal<R>(const double*, int, int, R*, int, int, int, const int32_t*, int64_t, int,        \
-                                      double, const double*, cudaStream_t);                                           \
-  template void launch_to_external<R>(const R*, int, int, double*, int, int, int, const int32_t*, int64_t, int,       \
-                                      cudaStream_t);                                                                  \
+  template void launch_to_internal<R>(int, const double*, const double*, int64_t, R*, const int32_t*, int64_t,         \
+                                      const double*, cudaStream_t);                                                   \
+  template void launch_to_external<R>(int, const R*, double*, double*, int64_t, const int32_t*, int64_t, cudaStream_t); \
   template void launch_lincomb3<R>(R*, R*, R*, double, const R*, double, const R*, int64_t, cudaStream_t);             \
   template void launch_lincomb3_masked<R>(R*, R*, R*, double, const R*, double, const R*, int64_t, int,                 \
                                           const int32_t*, const int32_t*, cudaStream_t);                                \
@@ -474,8 +577,7 @@ void launch_finalize(const double* partials, const BlockTable& bt, Scalars* sc, 
   template void launch_dot<R>(int, const R*, const R*, const double*, double*, const BlockTable&, cudaStream_t);      \
   template void launch_scatter_rows<R>(R*, R*, const double*, const double*, const int64_t*, int64_t, int,        \
                                        cudaStream_t);                                                              \
-  template void launch_set_gvol_item<R>(R*, int, const double*, const double*, const int32_t*, int64_t,             \
-                                        cudaStream_t);                                                             \
+  template void launch_set_sigma<R>(R*, const double*, const double*, const int32_t*, int64_t, cudaStream_t);        \
   template void launch_halo<R>(R*, const int64_t*, const int64_t*, int64_t, int, cudaStream_t);                        \
   template void launch_cg_direction<R>(R*, R*, const R*, const Scalars*, const int32_t*, const int32_t*, int64_t,     \
                                        int, cudaStream_t);
