@@ -85,31 +85,26 @@ __device__ __forceinline__ void cp_async_wait() {
 // - hcs[2h+1] J_im,h.  The even lane reads J_re and the odd lane J_im, as one line (jv: already read,
 // single frequency), and the odd lane, which computes Phi_E, adds both.
 template <typename R, int NN>
-__device__ __forceinline__ void load_source(R (&jv)[3][NN], const R* j, int n0) {
+__device__ __forceinline__ void load_source(R (&jv)[NN], const R* j, int c, int n0) {
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int n = 0; n < NN; ++n) jv[c][n] = j[(c * NPQ + n0 + n) * 32];
+  for (int n = 0; n < NN; ++n) jv[n] = j[(c * NPQ + n0 + n) * 32];
 }
 template <typename R, int NN>
-__device__ __forceinline__ void add_source(R (&phi)[3][NN], const R (&jv)[3][NN], R cs, R sn, int half) {
+__device__ __forceinline__ void add_source(R (&phi)[NN], const R (&jv)[NN], R cs, R sn, int half) {
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int n = 0; n < NN; ++n) {
-      const R re = __shfl_xor_sync(0xffffffffu, jv[c][n], 1);
-      if (half) phi[c][n] += cs * re - sn * jv[c][n];
-    }
+  for (int n = 0; n < NN; ++n) {
+    const R re = __shfl_xor_sync(0xffffffffu, jv[n], 1);
+    if (half) phi[n] += cs * re - sn * jv[n];
+  }
 }
+// Component c.
 template <typename R, int NN>
-__device__ __forceinline__ void add_data(R (&phi)[3][NN], const R (&jv)[3][NN], const StageArgs<R>& a,
-                                         const StageCoef<R>& cf, int64_t own, int n0, int half, R sigma) {
-  constexpr int NP = NPQ;
+__device__ __forceinline__ void add_data(R (&phi)[NN], const R (&jv)[NN], const StageArgs<R>& a, const StageCoef<R>& cf,
+                                         int64_t own, int c, int n0, int half, R sigma) {
+  const int64_t off = (own ^ 1) + (c * NPQ + n0) * 32;
   if (a.sigma && half) {  // Phi_E -= (sigma / eps) E (E is not flipped by Sigma)
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int n = 0; n < NN; ++n) phi[c][n] -= sigma * a.vin[(own ^ 1) + (c * NP + n0 + n) * 32];
+    for (int n = 0; n < NN; ++n) phi[n] -= sigma * a.vin[off + n * 32];
   }
   if (a.j) {
     if (a.nharm <= 0) {
@@ -117,47 +112,42 @@ __device__ __forceinline__ void add_data(R (&phi)[3][NN], const R (&jv)[3][NN], 
     } else {
 #pragma unroll 1
       for (int hh = 0; hh < a.nharm; ++hh) {
-        R jh[3][NN];
-        load_source<R, NN>(jh, a.j + hh * a.jstride + own, n0);
+        R jh[NN];
+        load_source<R, NN>(jh, a.j + hh * a.jstride + own, c, n0);
         add_source<R, NN>(phi, jh, a.hcs[2 * hh], a.hcs[2 * hh + 1], half);
       }
     }
   }
   if (a.bre) {  // impedance-face data, lifted (source sweeps only)
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int n = 0; n < NN; ++n) {
-        const int64_t o = (own ^ 1) + (c * NP + n0 + n) * 32;
-        phi[c][n] += cf.s_cos * a.bre[o] - cf.s_sin * a.bim[o];
-      }
+    for (int n = 0; n < NN; ++n) phi[n] += cf.s_cos * a.bre[off + n * 32] - cf.s_sin * a.bim[off + n * 32];
   }
 }
 
-// The on-the-fly filter on this thread's output values n0 .. n0 + NN - 1 (forward sweeps with
-// the filter, first nested stage of each step): F += fa U + fb Phi.  Each component's rows of U and
-// F are loaded before any of them is stored: vin, fre and fim are not known to be distinct, and a
+// The on-the-fly filter on component c of this thread's output values i0 .. i0 + NN - 1 (forward
+// sweeps with the filter, first nested stage of each step): F += fa U + fb Phi.  A batch of rows of
+// U and F is loaded before any of it is stored: vin, fre and fim are not known to be distinct, and a
 // row-by-row read-modify-write would put every load behind the previous row's stores.
 template <typename R, int NN>
-__device__ __forceinline__ void accumulate_filter(const StageArgs<R>& a, const StageCoef<R>& cf,
-                                                  const R (&phi)[3][NN], int64_t off, int n0) {
-  constexpr int NP = NPQ;
+__device__ __forceinline__ void accumulate_filter(const StageArgs<R>& a, const StageCoef<R>& cf, const R (&phi)[NN],
+                                                  int64_t own, int c, int i0) {
+  const int64_t off = (own ^ 1) + (c * NPQ + i0) * 32;
 #pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    R u[NN], fr[NN], fi[NN];
+  for (int n0 = 0; n0 < NN; n0 += 10) {  // ten rows at a time
+    R u[10], fr[10], fi[10];
 #pragma unroll
-    for (int ii = 0; ii < NN; ++ii) {
-      const int64_t o = off + (c * NP + n0 + ii) * 32;
-      u[ii] = a.vin[o];
-      fr[ii] = a.fre[o];
-      fi[ii] = a.fim[o];
-    }
+    for (int n = 0; n < 10; ++n)
+      if (n0 + n < NN) {
+        u[n] = a.vin[off + (n0 + n) * 32];
+        fr[n] = a.fre[off + (n0 + n) * 32];
+        fi[n] = a.fim[off + (n0 + n) * 32];
+      }
 #pragma unroll
-    for (int ii = 0; ii < NN; ++ii) {
-      const int64_t o = off + (c * NP + n0 + ii) * 32;
-      a.fre[o] = fr[ii] + (cf.fa_re * u[ii] + cf.fb_re * phi[c][ii]);
-      a.fim[o] = fi[ii] + (cf.fa_im * u[ii] + cf.fb_im * phi[c][ii]);
-    }
+    for (int n = 0; n < 10; ++n)
+      if (n0 + n < NN) {
+        a.fre[off + (n0 + n) * 32] = fr[n] + (cf.fa_re * u[n] + cf.fb_re * phi[n0 + n]);
+        a.fim[off + (n0 + n) * 32] = fi[n] + (cf.fa_im * u[n] + cf.fb_im * phi[n0 + n]);
+      }
   }
 }
 
@@ -239,11 +229,6 @@ constexpr size_t stage_smem() {
   if (sizeof(R) == 8) return SPLIT > 1 ? size_t(WARPS) * 3 * NPQ * 32 * sizeof(R) : 0;
   return size_t(WARPS) * nodal_smem<SPLIT>() * sizeof(R);
 }
-template <typename R>
-bool prefetches_source(const StageArgs<R>& a) {
-  return a.j != nullptr && a.nharm <= 0;
-}
-
 template <typename Arg>
 void launch_k(void (*k)(Arg), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s, bool pdl,
               const Arg& a) {
@@ -281,8 +266,7 @@ void launch_stage<CMCG_Q, float>(const StageArgs<float>& a, cudaStream_t s, int 
     case 4: launch_form<float, 2, 4, 4>(a, s, pdl); break;
     case 5: launch_form<float, 4, 4, 4>(a, s, pdl); break;
     case STAGE_FORM_TC:
-      launch_k(dg_stage_tc<TC_MINB>, unsigned((a.nti + TC_TETS - 1) / TC_TETS), TC_THREADS,
-               tc_smem(prefetches_source(a)), s, pdl, a);
+      launch_k(dg_stage_tc<TC_MINB>, unsigned((a.nti + TC_TETS - 1) / TC_TETS), TC_THREADS, tc_smem(), s, pdl, a);
       break;
     default: launch_form<float, 1, 4, 3>(a, s, pdl); break;
   }
@@ -307,7 +291,7 @@ void upload_constants<CMCG_Q>(const RefMats& rm) {
   allow_smem<float, 4, 4, 4>();
   allow_smem<double, 2, 2, 1>();
   allow_smem<double, 4, 4, 1>();
-  cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(tc_smem(true)));
+  cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(tc_smem()));
   cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributePreferredSharedMemoryCarveout,
                        int(cudaSharedmemCarveoutMaxShared));  // two P3 CTAs per SM need 2 x 113 KB
   tc_upload_reference(rm);

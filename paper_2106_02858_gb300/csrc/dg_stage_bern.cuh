@@ -170,7 +170,7 @@ __device__ __forceinline__ void bern_part(const StageArgs<double>& a, int64_t ht
     for (int n = 0; n < NP; ++n) phi[c][n] = double(0);
 #pragma unroll
   for (int m = P * NA / SPLIT; m < (P + 1) * NA / SPLIT; ++m) add_curl(phi, v, G, m);
-  double bv[3][NN], jv[3][NN];
+  double bv[3][NN];
 #pragma unroll
   for (int ff = 0; ff < NF; ++ff) {
     if (ff + 1 < NF) load_trace(tr[(ff + 1) & 1], a.vin, F[ff + 1].nb);
@@ -180,7 +180,6 @@ __device__ __forceinline__ void bern_part(const StageArgs<double>& a, int64_t ht
 #pragma unroll
         for (int n = 0; n < NN; ++n) bv[c][n] = a.base[(own ^ 1) + (c * NP + I0 + n) * 32];
     }
-    if (ff + 1 == NF && a.j && a.nharm <= 0) load_source<double, NN>(jv, a.j + own, I0);
     double g[2][NFPQ];
     bern_flux(g, tr[ff & 1], v, F[ff].t, F[ff].nb.c, F[ff].k, F0 + ff);
     add_lift(phi, g, F[ff].t, F[ff].k1, F0 + ff);
@@ -211,14 +210,16 @@ __device__ __forceinline__ void bern_part(const StageArgs<double>& a, int64_t ht
 #pragma unroll
       for (int n = 0; n < NN; ++n) out[c][n] = phi[c][n];
   }
-  add_data<double, NN>(out, jv, a, cf, own, I0, half, sigma);
-  if (a.fre) accumulate_filter<double, NN>(a, cf, out, own ^ 1, I0);  // forward sweeps with the filter only
-  if (a.out) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
+  for (int c = 0; c < 3; ++c) {
+    double jv[NN] = {};
+    if (a.j && a.nharm <= 0) load_source<double, NN>(jv, a.j + own, c, I0);
+    add_data<double, NN>(out[c], jv, a, cf, own, c, I0, half, sigma);
+    if (a.fre) accumulate_filter<double, NN>(a, cf, out[c], own, c, I0);  // forward sweeps with the filter only
+    if (a.out) {
 #pragma unroll
-      for (int n = 0; n < NN; ++n)
-        a.out[(own ^ 1) + (c * NP + I0 + n) * 32] = bv[c][n] + cf.c_out * out[c][n];
+      for (int n = 0; n < NN; ++n) a.out[(own ^ 1) + (c * NP + I0 + n) * 32] = bv[c][n] + cf.c_out * out[c][n];
+    }
   }
 }
 

@@ -149,7 +149,10 @@ __device__ __forceinline__ void nodal_part(const StageArgs<float>& a, int64_t ht
 #pragma unroll
           for (int n = 0; n < NN; ++n) bv[c][n] = a.base[(own ^ 1) + (c * NP + I0 + n) * 32];
       }
-      if (a.j && a.nharm <= 0) load_source<float, NN>(jv, a.j + own, I0);
+      if (a.j && a.nharm <= 0) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) load_source<float, NN>(jv[c], a.j + own, c, I0);
+      }
     }
     const int f = F0 + ff;
     float fl[3][NFP];
@@ -194,13 +197,13 @@ __device__ __forceinline__ void nodal_part(const StageArgs<float>& a, int64_t ht
       for (int n = 0; n < NN; ++n) bv[c][n] = gsm[GEO32 + (c * NP + n) * 32 + (l ^ 1)];
   }
   const float sigma = a.sigma ? gp[GEO_SIGMA * 32] : 0.0f;
-  add_data<float, NN>(phi, jv, a, cf, own, I0, half, sigma);
-  if (a.fre) accumulate_filter<float, NN>(a, cf, phi, own ^ 1, I0);  // forward sweeps with the filter only
-  if (a.out) {
 #pragma unroll
-    for (int c = 0; c < 3; ++c)
+  for (int c = 0; c < 3; ++c) {
+    add_data<float, NN>(phi[c], jv[c], a, cf, own, c, I0, half, sigma);
+    if (a.fre) accumulate_filter<float, NN>(a, cf, phi[c], own, c, I0);  // forward sweeps with the filter only
+    if (a.out) {
 #pragma unroll
-      for (int n = 0; n < NN; ++n)
-        a.out[(own ^ 1) + (c * NP + I0 + n) * 32] = bv[c][n] + cf.c_out * phi[c][n];
+      for (int n = 0; n < NN; ++n) a.out[(own ^ 1) + (c * NP + I0 + n) * 32] = bv[c][n] + cf.c_out * phi[c][n];
+    }
   }
 }

@@ -4,10 +4,10 @@
 // and the lift LIFT . f of the face fluxes.  FP32 sweeps only; included by
 // dg_stage.cuh inside its anonymous namespace, once per order.
 //
-// Mapping.  A CTA of 128 threads covers 64 tetrahedra (four half tiles, one per
-// warp); thread t is row t of every MMA and lane t of tensor memory (TMEM), and,
-// as in dg_stage_kernel, lanes 2k and 2k + 1 hold the electric and the magnetic
-// field of one tetrahedron (each computes the other field's Phi).  Per row:
+// Mapping.  A CTA covers 64 tetrahedra (four half tiles) with two warpgroups.  Row r of
+// every MMA (lane r of tensor memory, TMEM) belongs to threads r and 128 + r; as in
+// dg_stage_kernel, rows 2k and 2k + 1 hold the electric and the magnetic field of one
+// tetrahedron (each gives the other field's Phi).  Per row:
 //
 //   volume:  d_{c'}[(b, i)] = sum_j F_{c'}[j] D_b[i][j]      (3 MMAs chains, K = Np, N = 3 Np)
 //   lift:    L_c[i]        = sum_k f_c[k] LIFT[i][k]        (3 chains, K = 4 Nfp, N = Np)
@@ -27,44 +27,49 @@
 // (the lo_a lo_b term, ~2^-22 relative, is dropped), accumulated in FP32 in TMEM.
 // The reference matrices are split on the host from double (both parts rounded).
 //
-// Synchronisation.  One thread issues every MMA of the CTA; the six contractions
-// (volume of own components 0, 1, 2, then lift of output components 0, 1, 2) use
-// two TMEM buffers in turn, each with its own mbarrier, so that at most 256 TMEM
-// columns are held and two CTAs can share an SM.  All waits on mbarriers are bounded (about one second of
-// %globaltimer), after which the CTA records CMCG_ERR_DEVICE_TIMEOUT in a.err,
-// skips the dependent work, frees its TMEM and returns.  TMEM is allocated after
-// the grid-dependency wait, so a CTA that starts early under programmatic
-// dependent launch never holds TMEM while the previous stage still runs; the
-// bulk copy of the reference matrices is issued before that wait.
+// Warpgroup 0 (threads 0 to 127) runs the volume term: it writes the own field's operands,
+// reads the derivatives back and applies the chain rule and the curl.  Warpgroup 1 meanwhile
+// gathers the neighbour traces and computes the face fluxes, into shared memory.  Both write
+// the lift's operands; warpgroup 0 adds the lift to components 0 and 1 and writes their output,
+// warpgroup 1 component 2's.  One warpgroup doing all of this in turn took 10.2 us for a lone
+// CTA (one warp per scheduler issuing 4,200 dependent instructions, 18% of the issue slots) and
+// 13.3 us per stage of 12,288 P3 tetrahedra; two take 7.8 us and 12.0 us.
+//
+// An MMA takes 33 (N = 64) or 18 cycles (N = 32) when its operands are uniform registers of a
+// converged warp and one elected lane issues it; issued from a branch for one lane, whose registers
+// the hardware has to make uniform first, it took 118 and 61, more than everything else a warp does.
+//
+// Synchronisation.  The contractions run in four batches: volume of components 0 and 1, volume
+// of 2, lift of 0 and 1, lift of 2.  The warps that write a batch's operands arrive on its
+// rdy[], its MMAs are committed to its done[].  Volume component 2 uses component 0's columns
+// again; then, all derivatives being read and all fluxes computed (one barrier of the CTA), the
+// lift lays the columns out anew: three accumulators and two operands, component 2's in the
+// place of component 0's once that has been read.  256 columns are held, so two CTAs share an
+// SM.  All waits on mbarriers are bounded (about one second of %globaltimer), after which the
+// CTA records CMCG_ERR_DEVICE_TIMEOUT in a.err, skips the dependent work, frees its TMEM and
+// returns.  TMEM is allocated after the grid-dependency wait, so a CTA that starts early under
+// programmatic dependent launch never holds TMEM while the previous stage still runs; the bulk
+// copy of the reference matrices is issued before that wait.
 
-constexpr int TC_THREADS = 128;
+constexpr int TC_ROWS = 128;
+constexpr int TC_THREADS = 2 * TC_ROWS;
 constexpr int TC_TETS = 64;
 constexpr int TC_KV = (NPQ + 7) / 8 * 8;              // volume K (nodes), padded to the MMA K of 8
 constexpr int TC_KL = (4 * NFPQ + 7) / 8 * 8;         // lift K (face nodes f Nfp + jf)
-// Accumulator columns.  The output nodes are split in two halves of NH, each half's columns
-// one aligned block (a layout that lets a thread group own one node half):
-//   volume: column of (b, i) = h VBLK + b NH + (i - h NH), h = i / NH;   N = 2 VBLK
-//   lift:   column of i      = h LBLK + (i - h NH);                       N = 2 LBLK
-constexpr int TC_NH = NPQ / 2;
-constexpr int tc_pow2_at_least(int x) { return x <= 8 ? 8 : x <= 16 ? 16 : x <= 32 ? 32 : 64; }
-constexpr int TC_VBLK = tc_pow2_at_least(3 * TC_NH);
-constexpr int TC_LBLK = tc_pow2_at_least(TC_NH);
-constexpr int TC_NV = 2 * TC_VBLK;                    // volume N
-constexpr int TC_NL = 2 * TC_LBLK;                    // lift N
-static_assert(NPQ % 2 == 0 && TC_NV % 16 == 0 && TC_NL % 16 == 0, "accumulator blocks");
-__host__ __device__ constexpr int tc_vcol(int b, int i) {
-  return (i / TC_NH) * TC_VBLK + b * TC_NH + (i % TC_NH);
-}
-__host__ __device__ constexpr int tc_lcol(int i) { return (i / TC_NH) * TC_LBLK + (i % TC_NH); }
-// TMEM columns: two buffers of TC_BUF columns.  A buffer holds one component's
-// contraction: its accumulator [0, N) and its A operand, hi [N, N + K) and lo
-// [N + K, N + 2K) -- volume (N = NV, K = KV) or lift (N = NL, K = KL).  The six
-// contractions (3 volume, then 3 lift) alternate between the buffers, so one
-// component's MMAs run while the previous component's result is read.
-constexpr int TC_NEED = (TC_NV + 2 * TC_KV) > (TC_NL + 2 * TC_KL) ? (TC_NV + 2 * TC_KV) : (TC_NL + 2 * TC_KL);
-constexpr int TC_BUF = TC_NEED <= 32 ? 32 : TC_NEED <= 64 ? 64 : TC_NEED <= 128 ? 128 : 256;
-constexpr int TC_COLS = 2 * TC_BUF;
-static_assert(TC_COLS <= 256, "two CTAs per SM need at most 256 TMEM columns each");
+// Accumulator columns.  Volume: the derivatives of node i along b = 0, 1, 2 are neighbours, five
+// nodes to a block of 16 columns (one TMEM load).  Lift: column i.
+constexpr int TC_PER = NPQ < 5 ? NPQ : 5;
+constexpr int TC_NV = NPQ / TC_PER * 16;
+constexpr int TC_NL = (NPQ + 15) / 16 * 16;
+static_assert(NPQ % TC_PER == 0, "whole blocks");
+__host__ __device__ constexpr int tc_vcol(int b, int i) { return i / TC_PER * 16 + i % TC_PER * 3 + b; }
+// TMEM columns.  Volume: buffer b at b TC_COLS / 2, its accumulator [0, NV) and its operand, hi
+// [NV, NV + KV) and lo [NV + KV, NV + 2 KV).  Lift: accumulator of component c at c NL, operands 0
+// and 1 (hi, then lo, KL columns each) behind the accumulators; component 2 uses operand 0.
+constexpr int TC_LIFT_A = 3 * TC_NL;
+constexpr int TC_NEED = 2 * (TC_NV + 2 * TC_KV) > TC_LIFT_A + 4 * TC_KL ? 2 * (TC_NV + 2 * TC_KV) : TC_LIFT_A + 4 * TC_KL;
+constexpr int TC_COLS = TC_NEED <= 128 ? 128 : 256;
+static_assert(TC_NEED <= TC_COLS, "two CTAs per SM need at most 256 TMEM columns each");
 
 // Reference matrices for the MMAs (B operands), split hi / lo, in the core-matrix
 // layout: [BV hi | BV lo | BL hi | BL lo], BV = NV x KV, BL = NL x KL (row-major
@@ -123,11 +128,11 @@ __device__ __forceinline__ void tmem_ld16(uint32_t addr, float (&f)[16]) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
 
-// One MMA D[tmem d] (+)= A[tmem a] B[smem desc b]^T, M = 128.
+// One MMA D[tmem d] (+)= A[tmem a] B[smem desc b]^T, M = 128, by one elected lane of a converged warp.
 __device__ __forceinline__ void tc_mma(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
   asm volatile(
-      "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+      "{\n.reg .pred p, e;\nelect.sync _|e, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"
+      "@e tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
       "r"(a), "l"(b), "r"(idesc), "r"(accumulate)
       : "memory");
 }
@@ -153,24 +158,91 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   }
 }
 
+// Reductions over the CTA (its warps arrive from their own code paths).
+__device__ __forceinline__ bool cta_and(bool x) {
+  uint32_t r;
+  asm volatile(
+      "{\n.reg .pred p, q;\nsetp.ne.u32 p, %1, 0;\nbarrier.cta.red.and.pred q, 3, %2, p;\nselp.u32 %0, 1, 0, q;\n}\n"
+      : "=r"(r)
+      : "r"(uint32_t(x)), "n"(TC_THREADS)
+      : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ bool cta_or(bool x) { return !cta_and(!x); }
+
+// Zero-padded K-column operand at TMEM address addr, split hi / lo: value k is val(k) for k < n.
+// Columns [K0, K1) of it.
+template <int K, int K0, int K1, typename Val>
+__device__ __forceinline__ void tc_store_operand(uint32_t addr, int n, Val&& val) {
+#pragma unroll
+  for (int k0 = K0; k0 < K1; k0 += 8) {
+    uint32_t hi[8], lo[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      if (k0 + k < n) {
+        tf32_split(val(k0 + k), hi[k], lo[k]);
+      } else {
+        hi[k] = 0u;
+        lo[k] = 0u;
+      }
+    }
+    tmem_st8(addr + k0, hi);
+    tmem_st8(addr + K + k0, lo);
+  }
+}
+
+// The MMAs of NC contractions in turn (one warp): D = A_lo B_hi + A_hi B_lo + A_hi B_hi over the K
+// steps, then a commit to the mbarrier `bar` (also when skipped, so that waiters are released).
+// Contraction x: accumulator d + x dd, operand hi ahi + x da; bhi: shared address of the B operand's
+// hi part, its lo part blo bytes behind.
+template <int K, int NC>
+__device__ __forceinline__ void tc_issue(uint32_t d, uint32_t dd, uint32_t ahi, uint32_t da, uint32_t b, uint32_t blo,
+                                         uint32_t idesc, uint32_t bar, bool go) {
+  if (go) {
+    constexpr uint32_t sbo = uint32_t(K / 4) * 128;
+#pragma unroll
+    for (int s = 0; s < K / 8; ++s) {
+      const uint64_t bh = tc_desc(b + 256 * s, 128, sbo), bl = tc_desc(b + blo + 256 * s, 128, sbo);
+#pragma unroll
+      for (int x = 0; x < NC; ++x) tc_mma(d + x * dd, ahi + x * da + K + 8 * s, bh, idesc, s > 0 ? 1u : 0u);
+#pragma unroll
+      for (int x = 0; x < NC; ++x) tc_mma(d + x * dd, ahi + x * da + 8 * s, bl, idesc, 1u);
+#pragma unroll
+      for (int x = 0; x < NC; ++x) tc_mma(d + x * dd, ahi + x * da + 8 * s, bh, idesc, 1u);
+    }
+  }
+  asm volatile(
+      "{\n.reg .pred e;\nelect.sync _|e, 0xffffffff;\n"
+      "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar)
+      : "memory");
+}
+
+// The warp's part of an operand is written (and its reads of the accumulator are done).
+__device__ __forceinline__ void tc_ready(uint32_t bar) {
+  asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
+  tc_fence_before();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(bar) : "memory");
+}
+
 template <int MINB>
 __global__ void __launch_bounds__(TC_THREADS, MINB) dg_stage_tc(const StageArgs<float> a) {
   using R = float;
   constexpr int NP = NPQ, NFP = NFPQ;
   constexpr FaceTab FM = make_fmask(CMCG_Q);
-  constexpr uint32_t IDV = tc_idesc(128, TC_NV), IDL = tc_idesc(128, TC_NL);
+  constexpr int KM = (TC_KL / 8 + 1) / 2 * 8;  // lift operand columns written by warpgroup 0, the rest by 1
   grid_dep_launch();
-  const int tid = threadIdx.x, warp = tid >> 5, l = tid & 31, half = l & 1;
-  const int64_t ht = int64_t(blockIdx.x) * (TC_THREADS / 32) + warp;
+  const int tid = threadIdx.x, wg = tid >> 7, row = tid & 127, warp = row >> 5, l = tid & 31, half = l & 1;
+  const int64_t ht = int64_t(blockIdx.x) * (TC_ROWS / 32) + warp;
   const bool in_range = ht * HTILE < a.nti;  // warp-uniform
 
-  __shared__ __align__(8) uint64_t bars[3];  // [0]: reference matrices loaded, [1 + b]: MMAs of buffer b
+  // Batches 0, 1: volume of own components 0 and 1, then 2; 2, 3: lift of output components 0 and 1, then 2.
+  __shared__ __align__(8) uint64_t bars[9];  // reference matrices; rdy[4]; done[4]
   __shared__ uint32_t tmem_base;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  unsigned char* sB = smem_raw;                                            // TC_B_BYTES
-  R* tr = reinterpret_cast<R*>(smem_raw + TC_B_BYTES) + tid;               // trace / flux slots
-  R* bs = tr + 4 * NFP * 3 * TC_THREADS;                                   // base rows
-  R* js = bs + 3 * NP * TC_THREADS;  // source rows (single-frequency source stages)
+  unsigned char* sB = smem_raw;                               // TC_B_BYTES
+  R* fl = reinterpret_cast<R*>(smem_raw + TC_B_BYTES) + row;  // traces, then fluxes: component c of face node k at (c 4 Nfp + k) TC_ROWS
+  R* ph = fl + 4 * NFP * 3 * TC_ROWS;                         // the volume term of component 2
   const bool jpre = a.j && a.nharm <= 0;
 
   int prob = 0;
@@ -181,311 +253,281 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) dg_stage_tc(const StageArgs<
     cf = a.coef[prob];
   }
   bool live = in_range && cf.active;
-  if (!__syncthreads_or(live)) return;  // CTA-uniform
-  // A warp without a half tile takes half tile 0's geometry and neighbours, and stores nothing.
-  const int64_t hr = in_range ? ht : 0;
-  R G[9];
-#pragma unroll
-  for (int m = 0; m < 9; ++m) G[m] = a.geo[hr * GEO32 + m * 16 + (l >> 1)];
-  const R sv = a.geo[hr * GEO32 + GEO_S32 * 16 + l] * a.sH;
-  struct Face {
-    R n[3], k1, k2;
-    Neighbour<R> nb;
-  } F[4];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) F[f].n[k] = a.geo[hr * GEO32 + (9 + 3 * f + k) * 16 + (l >> 1)];
-    const R* gp = a.geo + hr * GEO32 + GEO_S32 * 16 + (1 + 2 * f) * 32 + l;
-    F[f].k1 = gp[0] * a.sH;
-    F[f].k2 = gp[32];
-    F[f].nb = find_neighbour(a, hr, l, f);
-  }
-  const R sigma = a.sigma ? a.geo[hr * GEO32 + (GEO_S32 * 16 + GEO_SIGMA * 32) + l] : R(0);
+  if (!cta_or(live)) return;  // CTA-uniform
+  const uint32_t barB = smem_addr(&bars[0]), rdy = smem_addr(&bars[1]), done = smem_addr(&bars[5]);
+  const uint32_t sb = smem_addr(sB);
   // The reference matrices (written only at handle creation) are copied before the grid
   // dependency: one bulk copy, completion counted in bytes on barB.
-  const uint32_t barB = smem_addr(&bars[0]);
-  const uint32_t barM[2] = {smem_addr(&bars[1]), smem_addr(&bars[2])};
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(barB));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(barM[0]));
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(barM[1]));
+#pragma unroll
+    for (int x = 0; x < 4; ++x) {
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(rdy + 8 * x), "r"(x < 2 ? 4 : 8));
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(done + 8 * x));
+    }
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(barB), "r"(TC_B_BYTES) : "memory");
     asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-            smem_addr(sB)),
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(sb),
         "l"(gTcB), "r"(TC_B_BYTES), "r"(barB)
         : "memory");
   }
-  grid_dep_wait();
-  if (live && a.pactive && !a.pactive[prob]) live = false;  // CG converged (written by the CG kernels)
-  if (!__syncthreads_or(live)) {
-    if (tid == 0) mbar_wait(barB, 0);  // the copy lands before the CTA's shared memory is released
+
+  // A warp without a half tile takes half tile 0's geometry and neighbours, and stores nothing.
+  const int64_t hr = in_range ? ht : 0;
+  const int64_t own = hr * HS + l;  // the thread's field; its output is the partner's, own ^ 1
+  const R* gs = a.geo + hr * GEO32 + (l >> 1);
+  const R* gp = a.geo + hr * GEO32 + GEO_S32 * 16 + l;
+  uint32_t tmem = 0, trow = 0;  // this CTA's columns, this warp's lanes of them
+  // Batch x's MMAs, by the warp that calls this (all operands warp-uniform).
+  auto issue = [&](int x, bool ok) -> bool {
+    ok = mbar_wait(barB, 0) && ok;
+    ok = mbar_wait(rdy + 8 * x, 0) && ok;
+    tc_fence_after();
+    const bool go = __all_sync(0xffffffffu, ok);
+    const uint32_t t = __shfl_sync(0xffffffffu, tmem, 0);
+    constexpr uint32_t IV = tc_idesc(128, TC_NV), IL = tc_idesc(128, TC_NL), H = TC_COLS / 2, SL = 2 * TC_BV_BYTES;
+    if (x == 0) tc_issue<TC_KV, 2>(t, H, t + TC_NV, H, sb, TC_BV_BYTES, IV, done + 8 * x, go);
+    if (x == 1) tc_issue<TC_KV, 1>(t, 0, t + TC_NV, 0, sb, TC_BV_BYTES, IV, done + 8 * x, go);
+    if (x == 2) tc_issue<TC_KL, 2>(t, TC_NL, t + TC_LIFT_A, 2 * TC_KL, sb + SL, TC_BL_BYTES, IL, done + 8 * x, go);
+    if (x == 3) tc_issue<TC_KL, 1>(t + 2 * TC_NL, 0, t + TC_LIFT_A, 0, sb + SL, TC_BL_BYTES, IL, done + 8 * x, go);
+    return ok;
+  };
+  const bool first = __shfl_sync(0xffffffffu, warp, 0) == 0;  // the warpgroup's first warp
+  // Columns of the lift operand of component c (value k: flux k of the row), the warpgroup's share.
+  auto store_lift = [&](int c) {
+    const uint32_t addr = trow + TC_LIFT_A + (c == 1 ? 2 * TC_KL : 0);
+    auto flux = [&](int k) { return fl[(c * 4 * NFP + k) * TC_ROWS]; };
+    if (wg == 0) tc_store_operand<TC_KL, 0, KM>(addr, 4 * NFP, flux);
+    else tc_store_operand<TC_KL, KM, TC_KL>(addr, 4 * NFP, flux);
+  };
+  // Component c: the lift added to the volume term p, data, filter, output.
+  auto finish = [&](int c, R (&p)[NP], const R (&bv)[NP], const R (&jv)[NP], R sigma) {
+#pragma unroll
+    for (int k0 = 0; k0 < TC_NL; k0 += 16) {
+      float t16[16];
+      tmem_ld16(trow + c * TC_NL + k0, t16);
+#pragma unroll
+      for (int i = 0; i < NP; ++i)
+        if (i / 16 * 16 == k0) p[i] += t16[i % 16];
+    }
+    if (!live) return;  // warp-uniform
+    add_data<R, NP>(p, jv, a, cf, own, c, 0, half, sigma);
+    if (a.fre) accumulate_filter<R, NP>(a, cf, p, own, c, 0);  // forward sweeps with the filter only
+    if (a.out) {
+#pragma unroll
+      for (int n = 0; n < NP; ++n) a.out[(own ^ 1) + (c * NP + n) * 32] = bv[n] + cf.c_out * p[n];
+    }
+  };
+  auto load_base = [&](R (&bv)[NP], int c) {
+    if (a.out) {
+#pragma unroll
+      for (int n = 0; n < NP; ++n) bv[n] = a.base[(own ^ 1) + (c * NP + n) * 32];
+    }
+  };
+  // Both warpgroups: fluxes computed, derivatives read.
+  auto middle = [&]() {
+    tc_fence_before();
+    asm volatile("barrier.cta.sync 1, 256;\n" ::: "memory");
+    tc_fence_after();
+  };
+
+  if (wg == 1) {
+    // ---- warpgroup 1: neighbour traces, face fluxes
+    Neighbour<R> nb[4];
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      nb[f] = find_neighbour(a, hr, l, f);
+      asm volatile("" : "+l"(nb[f].at), "+l"(nb[f].nodes));  // looked up before the wait
+    }
+    grid_dep_wait();
+    if (live && a.pactive && !a.pactive[prob]) live = false;  // CG converged (written by the CG kernels)
+    if (!cta_or(live)) return;
+    // Traces of a face two faces ahead of its fluxes, each face a group of copies.
+    auto copy_face = [&](int f) {
+      const R* p = a.vin + nb[f].at;
+#pragma unroll
+      for (int jf = 0; jf < NFP; ++jf) {
+        const R* q = p + (unsigned(nb[f].nodes >> (5 * jf)) & 31u) * 32u;
+#pragma unroll
+        for (int c = 0; c < 3; ++c) cp_async_4(fl + (c * 4 * NFP + f * NFP + jf) * TC_ROWS, q + c * NP * 32);
+      }
+      cp_async_commit();
+    };
+    copy_face(0);
+    R v[3][NP];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+#pragma unroll
+      for (int n = 0; n < NP; ++n) v[c][n] = a.vin[own + (c * NP + n) * 32];
+    copy_face(1);
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+      if (f < 3) cp_async_wait<1>();
+      else cp_async_wait<0>();
+      if (f + 2 < 4) copy_face(f + 2 < 4 ? f + 2 : 0);
+      const R n0 = gs[(9 + 3 * f) * 16], n1 = gs[(10 + 3 * f) * 16], n2 = gs[(11 + 3 * f) * 16];
+      const R k1 = gp[(1 + 2 * f) * 32] * a.sH, k2 = gp[(2 + 2 * f) * 32];
+      const R m0 = k1 * n0, m1 = k1 * n1, m2 = k1 * n2;  // k1 n, once per face
+#pragma unroll
+      for (int g = 0; g < NFP; g += 5) {  // five nodes at a time: independent chains
+        R X[3][5], Y[3][5];
+#pragma unroll
+        for (int j = 0; j < 5; ++j)
+          if (g + j < NFP)
+#pragma unroll
+            for (int c = 0; c < 3; ++c)
+              X[c][j] = fmaf(nb[f].c, fl[(c * 4 * NFP + f * NFP + g + j) * TC_ROWS], -v[c][FM.v[f][g + j]]);
+#pragma unroll
+        for (int j = 0; j < 5; ++j)
+          if (g + j < NFP)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) Y[c][j] = __shfl_xor_sync(0xffffffffu, X[c][j], 1);
+#pragma unroll
+        for (int j = 0; j < 5; ++j)
+          if (g + j < NFP) {
+            const R nY = n0 * Y[0][j] + n1 * Y[1][j] + n2 * Y[2][j];
+            R* s = fl + (f * NFP + g + j) * TC_ROWS;
+            s[0 * 4 * NFP * TC_ROWS] = (m1 * X[2][j] - m2 * X[1][j]) + k2 * (Y[0][j] - n0 * nY);
+            s[1 * 4 * NFP * TC_ROWS] = (m2 * X[0][j] - m0 * X[2][j]) + k2 * (Y[1][j] - n1 * nY);
+            s[2 * 4 * NFP * TC_ROWS] = (m0 * X[1][j] - m1 * X[0][j]) + k2 * (Y[2][j] - n2 * nY);
+          }
+      }
+    }
+    middle();
+    tmem = tmem_base;
+    trow = tmem + (uint32_t(warp * 32) << 16);
+    store_lift(0);
+    store_lift(1);
+    tc_ready(rdy + 8 * 2);
+    R bv[NP];
+    load_base(bv, 2);
+    bool ok = true;
+    if (first) ok = issue(2, ok);
+    ok = mbar_wait(done + 8 * 2, 0) && ok;  // component 0's operand has been read
+    tc_fence_after();
+    store_lift(2);
+    tc_ready(rdy + 8 * 3);
+    if (first) ok = issue(3, ok);
+    R p[NP], jv[NP];
+    if (jpre) load_source<R, NP>(jv, a.j + own, 2, 0);
+#pragma unroll
+    for (int n = 0; n < NP; ++n) p[n] = ph[n * TC_ROWS];
+    ok = mbar_wait(done + 8 * 3, 0) && ok;
+    tc_fence_after();
+    if (ok) finish(2, p, bv, jv, a.sigma ? gp[GEO_SIGMA * 32] : R(0));
+    tc_fence_before();
+    cta_and(ok);
     return;
   }
 
+  // ---- warpgroup 0: volume, output
+  R G[9];
+  const R sv = gp[0] * a.sH;
+#pragma unroll
+  for (int m = 0; m < 9; ++m) G[m] = gs[m * 16] * sv;  // the material factor of Phi, folded into the chain rule
+  const R sigma = a.sigma ? gp[GEO_SIGMA * 32] : R(0);
+  grid_dep_wait();
+  if (live && a.pactive && !a.pactive[prob]) live = false;
+  if (!cta_or(live)) {
+    if (tid == 0) mbar_wait(barB, 0);  // the copy lands before the CTA's shared memory is released
+    return;
+  }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_addr(&tmem_base)),
                  "r"(TC_COLS));
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;\n");
   }
-
-  // Own field, neighbour traces, base rows and (single-frequency source stages) source rows.
-  R v[3][NP];
-  const int64_t own = hr * HS + l;  // the thread's field; its output is the partner's, own ^ 1
+  R v[2][NP];  // the own field, component 2 in place of component 0's
+  auto load_own = [&](int b, int c) {
 #pragma unroll
-  for (int c = 0; c < 3; ++c)
-#pragma unroll
-    for (int n = 0; n < NP; ++n) v[c][n] = a.vin[own + (c * NP + n) * 32];
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    const R* nb = a.vin + F[f].nb.at;
-#pragma unroll
-    for (int jf = 0; jf < NFP; ++jf) {
-      const R* p = nb + (unsigned(F[f].nb.nodes >> (5 * jf)) & 31u) * 32u;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) cp_async_4(tr + ((f * NFP + jf) * 3 + c) * TC_THREADS, p + c * NP * 32);
-    }
-  }
-  if (a.out) {
-#pragma unroll
-    for (int k = 0; k < 3 * NP; ++k) cp_async_4(bs + k * TC_THREADS, a.base + (own ^ 1) + k * 32);
-  }
-  if (jpre) {
-#pragma unroll
-    for (int k = 0; k < 3 * NP; ++k) cp_async_4(js + k * TC_THREADS, a.j + own + k * 32);
-  }
-  cp_async_commit();
-
+    for (int n = 0; n < NP; ++n) v[b][n] = a.vin[own + (c * NP + n) * 32];
+  };
+  load_own(0, 0);
+  load_own(1, 1);
   tc_fence_before();
-  __syncthreads();  // TMEM address and mbarrier initialisation visible
+  asm volatile("barrier.cta.sync 2, 128;\n" ::: "memory");  // TMEM address and mbarrier initialisation visible
   tc_fence_after();
-  const uint32_t tmem = tmem_base;
-  const uint32_t trow = tmem + (uint32_t(warp * 32) << 16);  // this warp's TMEM lanes
+  tmem = tmem_base;
+  trow = tmem + (uint32_t(warp * 32) << 16);
 
-  const uint32_t sb = smem_addr(sB);
-  // Volume A of component c into buffer b: the own field, split hi / lo, zero-padded to KV columns.
-  auto store_vol_a = [&](int b, int c) {
-#pragma unroll
-    for (int k0 = 0; k0 < TC_KV; k0 += 8) {
-      uint32_t hi[8], lo[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        if (k0 + k < NP) {
-          tf32_split(v[c][k0 + k], hi[k], lo[k]);
-        } else {
-          hi[k] = 0u;
-          lo[k] = 0u;
-        }
-      }
-      tmem_st8(trow + b * TC_BUF + TC_NV + k0, hi);
-      tmem_st8(trow + b * TC_BUF + TC_NV + TC_KV + k0, lo);
-    }
-  };
-  // Lift A of output component c into buffer b: the face fluxes (in the trace slots), split.
-  auto store_lift_a = [&](int b, int c) {
-#pragma unroll
-    for (int k0 = 0; k0 < TC_KL; k0 += 8) {
-      uint32_t hi[8], lo[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        if (k0 + k < 4 * NFP) {
-          tf32_split(tr[((k0 + k) * 3 + c) * TC_THREADS], hi[k], lo[k]);
-        } else {
-          hi[k] = 0u;
-          lo[k] = 0u;
-        }
-      }
-      tmem_st8(trow + b * TC_BUF + TC_NL + k0, hi);
-      tmem_st8(trow + b * TC_BUF + TC_NL + TC_KL + k0, lo);
-    }
-  };
-  // MMAs of buffer b (thread 0): D = A_lo B_hi + A_hi B_lo + A_hi B_hi over the K steps,
-  // then a commit to the buffer's mbarrier (also when skipped, so that waiters are released).
-  auto issue = [&](int b, bool lift, bool go) {
-    if (go) {
-      const uint32_t d = tmem + b * TC_BUF;
-      const uint32_t nacc = lift ? TC_NL : TC_NV;
-      const int K = lift ? TC_KL : TC_KV;
-      const uint32_t b0 = sb + (lift ? 2 * TC_BV_BYTES : 0);
-      const uint32_t blo_off = lift ? TC_BL_BYTES : TC_BV_BYTES;
-      const uint32_t sbo = uint32_t(K / 4) * 128;
-      const uint32_t idesc = lift ? IDL : IDV;
-#pragma unroll 1
-      for (int s8 = 0; s8 < K / 8; ++s8) {
-        const uint32_t ahi = d + nacc + 8 * s8, alo = ahi + K;
-        const uint64_t bhi = tc_desc(b0 + 256 * s8, 128, sbo);
-        const uint64_t blo = tc_desc(b0 + blo_off + 256 * s8, 128, sbo);
-        tc_mma(d, alo, bhi, idesc, s8 > 0 ? 1u : 0u);
-        tc_mma(d, ahi, blo, idesc, 1u);
-        tc_mma(d, ahi, bhi, idesc, 1u);
-      }
-    }
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(barM[b])
-                 : "memory");
-  };
-  // All A operands written and all accumulator reads done before thread 0 issues MMAs.
-  auto handoff = [&](bool ok_in) -> bool {
-    asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-    tc_fence_before();
-    const bool r = __syncthreads_and(ok_in);
-    tc_fence_after();
-    return r;
-  };
   R phi[3][NP];
 #pragma unroll
   for (int c = 0; c < 3; ++c)
 #pragma unroll
     for (int i = 0; i < NP; ++i) phi[c][i] = R(0);
   // Volume result of own component cp (buffer b): derivatives along r, s, t, chain rule, curl.
-#pragma unroll
-  for (int m = 0; m < 9; ++m) G[m] *= sv;  // the material factor of Phi, folded into the chain rule
   auto read_vol = [&](int b, int cp) {
-    float d[TC_NV];
-#pragma unroll
-    for (int k0 = 0; k0 < TC_NV; k0 += 16) {
-      float t16[16];
-      tmem_ld16(trow + b * TC_BUF + k0, t16);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) d[k0 + k] = t16[k];
-    }
     // curl F: component 0 = d1 F2 - d2 F1, 1 = d2 F0 - d0 F2, 2 = d0 F1 - d1 F0
     const int ap = cp == 0 ? 2 : cp == 1 ? 0 : 1;   // axis whose derivative enters with +
     const int am = cp == 0 ? 1 : cp == 1 ? 2 : 0;   // axis whose derivative enters with -
     const int cpl = cp == 0 ? 1 : cp == 1 ? 2 : 0;  // output component receiving + d_ap F_cp
     const int cmi = cp == 0 ? 2 : cp == 1 ? 0 : 1;  // output component receiving - d_am F_cp
-    // (G carries the material factor sv; each derivative is accumulated into Phi as an FMA chain)
 #pragma unroll
-    for (int i = 0; i < NP; ++i) {
-      const R d0 = d[tc_vcol(0, i)], d1 = d[tc_vcol(1, i)], d2 = d[tc_vcol(2, i)];
-      phi[cpl][i] = fmaf(G[2 * 3 + ap], d2, fmaf(G[1 * 3 + ap], d1, fmaf(G[0 * 3 + ap], d0, phi[cpl][i])));
-      phi[cmi][i] = fmaf(-G[2 * 3 + am], d2, fmaf(-G[1 * 3 + am], d1, fmaf(-G[0 * 3 + am], d0, phi[cmi][i])));
+    for (int i0 = 0; i0 < NP; i0 += TC_PER) {
+      float d[16];
+      tmem_ld16(trow + b * (TC_COLS / 2) + tc_vcol(0, i0), d);
+#pragma unroll
+      for (int i = i0; i < i0 + TC_PER; ++i) {
+        const R d0 = d[3 * (i - i0)], d1 = d[3 * (i - i0) + 1], d2 = d[3 * (i - i0) + 2];
+        phi[cpl][i] = fmaf(G[2 * 3 + ap], d2, fmaf(G[1 * 3 + ap], d1, fmaf(G[0 * 3 + ap], d0, phi[cpl][i])));
+        phi[cmi][i] = fmaf(-G[2 * 3 + am], d2, fmaf(-G[1 * 3 + am], d1, fmaf(-G[0 * 3 + am], d0, phi[cmi][i])));
+      }
     }
   };
-  auto read_lift = [&](int b, int c) {
-    float l[TC_NL];
-#pragma unroll
-    for (int k0 = 0; k0 < TC_NL; k0 += 16) {
-      float t16[16];
-      tmem_ld16(trow + b * TC_BUF + k0, t16);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) l[k0 + k] = t16[k];
-    }
-#pragma unroll
-    for (int i = 0; i < NP; ++i) phi[c][i] += l[tc_lcol(i)];
+  auto store_vol = [&](int b) {
+    tc_store_operand<TC_KV, 0, TC_KV>(trow + b * (TC_COLS / 2) + TC_NV, NP, [&](int k) { return v[b][k]; });
   };
-
-  // Volume contractions of components 0 and 1 (buffers 0, 1).
-  store_vol_a(0, 0);
-  store_vol_a(1, 1);
-  asm volatile("tcgen05.wait::st.sync.aligned;\n" ::: "memory");
-  tc_fence_before();
-  __syncthreads();
-  bool okB = true;  // thread 0: the reference matrices arrived
-  if (tid == 0) {
-    tc_fence_after();
-    okB = mbar_wait(barB, 0);
-    issue(0, false, okB);
-    issue(1, false, okB);
-  }
-
-  // Face fluxes (CUDA cores, overlapping the volume MMAs), stored over the trace slots.
-  cp_async_wait<0>();
-#pragma unroll
-  for (int f = 0; f < 4; ++f) {
-    const R n0 = F[f].n[0], n1 = F[f].n[1], n2 = F[f].n[2], k2 = F[f].k2;
-    const R m0 = F[f].k1 * n0, m1 = F[f].k1 * n1, m2 = F[f].k1 * n2;  // k1 n, once per face
-#pragma unroll
-    for (int jf = 0; jf < NFP; ++jf) {
-      const int own_node = FM.v[f][jf];
-      R X[3], Y[3];
-#pragma unroll
-      for (int c = 0; c < 3; ++c) X[c] = fmaf(F[f].nb.c, tr[((f * NFP + jf) * 3 + c) * TC_THREADS], -v[c][own_node]);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) Y[c] = __shfl_xor_sync(0xffffffffu, X[c], 1);
-      const R nY = n0 * Y[0] + n1 * Y[1] + n2 * Y[2];
-      tr[((f * NFP + jf) * 3 + 0) * TC_THREADS] = (m1 * X[2] - m2 * X[1]) + k2 * (Y[0] - n0 * nY);
-      tr[((f * NFP + jf) * 3 + 1) * TC_THREADS] = (m2 * X[0] - m0 * X[2]) + k2 * (Y[1] - n1 * nY);
-      tr[((f * NFP + jf) * 3 + 2) * TC_THREADS] = (m0 * X[1] - m1 * X[0]) + k2 * (Y[2] - n2 * nY);
-    }
-  }
-
-  // Component 0's result, then component 2 into buffer 0; components 1 and 2's results.
-  // Buffer 0 completes phases 0, 1 (volume) and 2, 3 (lift), buffer 1 phases 0 and 1.
-  bool ok = mbar_wait(barM[0], 0);
-  ok = __syncthreads_and(ok && okB);
+  store_vol(0);
+  store_vol(1);
+  tc_ready(rdy + 8 * 0);
+  load_own(0, 2);
+  bool ok = true;
+  if (first) ok = issue(0, ok);
+  ok = mbar_wait(done + 8 * 0, 0) && ok;
   tc_fence_after();
+  store_vol(0);  // the operand has been read; the accumulator is read before the next MMAs are issued
   if (ok) read_vol(0, 0);
-  store_vol_a(0, 2);
-  ok = handoff(ok);
-  if (tid == 0) issue(0, false, ok);
-  ok = mbar_wait(barM[1], 0) && ok;
-  tc_fence_after();
+  tc_ready(rdy + 8 * 1);
+  if (first) ok = issue(1, ok);
   if (ok) read_vol(1, 1);
-  ok = mbar_wait(barM[0], 1) && ok;
+  ok = mbar_wait(done + 8 * 1, 0) && ok;
   tc_fence_after();
-  if (ok) {
-    read_vol(0, 2);
-  }
+  if (ok) read_vol(0, 2);
+#pragma unroll
+  for (int n = 0; n < NP; ++n) ph[n * TC_ROWS] = phi[2][n];
 
-  // Lift contractions: output components 0 and 1 (buffers 0, 1), then 2 into buffer 0.
-  store_lift_a(0, 0);
-  store_lift_a(1, 1);
-  ok = handoff(ok);
-  if (tid == 0) {
-    issue(0, true, ok);
-    issue(1, true, ok);
+  middle();
+  store_lift(0);
+  store_lift(1);
+  tc_ready(rdy + 8 * 2);
+  R bv[2][NP];
+  load_base(bv[0], 0);
+  load_base(bv[1], 1);
+  R jv[NP];
+  if (jpre) load_source<R, NP>(jv, a.j + own, 0, 0);
+  ok = mbar_wait(done + 8 * 2, 0) && ok;
+  tc_fence_after();
+  store_lift(2);
+  tc_ready(rdy + 8 * 3);
+  if (ok) {
+    finish(0, phi[0], bv[0], jv, sigma);
+    if (jpre) load_source<R, NP>(jv, a.j + own, 1, 0);
+    finish(1, phi[1], bv[1], jv, sigma);
   }
-  ok = mbar_wait(barM[0], 0) && ok;
-  tc_fence_after();
-  if (ok) read_lift(0, 0);
-  store_lift_a(0, 2);
-  ok = handoff(ok);
-  if (tid == 0) issue(0, true, ok);
-  ok = mbar_wait(barM[1], 1) && ok;
-  tc_fence_after();
-  if (ok) read_lift(1, 1);
-  ok = mbar_wait(barM[0], 1) && ok;
-  tc_fence_after();
-  if (ok) read_lift(0, 2);
   // Free TMEM (every thread's TMEM reads are complete).
   tc_fence_before();
-  ok = __syncthreads_and(ok);
+  ok = cta_and(ok);
   if (warp == 0) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem), "r"(TC_COLS));
   }
-  if (!ok) {
-    if (tid == 0 && a.err) atomicOr(a.err, 1);
-    return;
-  }
-  if (!live) return;
-
-  R jv[3][NP];
-  if (jpre) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int n = 0; n < NP; ++n) jv[c][n] = js[(c * NP + n) * TC_THREADS];
-  }
-  add_data<R, NP>(phi, jv, a, cf, own, 0, half, sigma);
-  if (a.fre) accumulate_filter<R, NP>(a, cf, phi, own ^ 1, 0);  // forward sweeps with the filter only
-  if (a.out) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c)
-#pragma unroll
-      for (int n = 0; n < NP; ++n)
-        a.out[(own ^ 1) + (c * NP + n) * 32] = bs[(c * NP + n) * TC_THREADS] + cf.c_out * phi[c][n];
-  }
+  if (!ok && tid == 0 && a.err) atomicOr(a.err, 1);
 }
 
-// Dynamic shared memory of dg_stage_tc: reference matrices, trace slots, base rows,
-// and the prefetched source rows of single-frequency source stages (src = true; J_re in the even
-// threads' slots, J_im in the odd ones').
-constexpr size_t tc_smem(bool src) {
-  return size_t(TC_B_BYTES) + size_t(4 * NFPQ * 3 + (src ? 6 : 3) * NPQ) * TC_THREADS * sizeof(float);
-}
+// Dynamic shared memory of dg_stage_tc: reference matrices, traces / fluxes, the volume term of
+// component 2.
+constexpr size_t tc_smem() { return size_t(TC_B_BYTES) + size_t(4 * NFPQ * 3 + NPQ) * TC_ROWS * sizeof(float); }
 // Resident CTAs per SM that the TMEM columns allow (512 per SM).
 constexpr int TC_MINB = 2;
 
@@ -513,6 +555,6 @@ void tc_upload_reference(const RefMats& rm) {
     for (int i = 0; i < np; ++i)
       for (int j = 0; j < np; ++j) put(0, tc_vcol(b, i), j, TC_KV, (*D[b])[size_t(i) * np + j]);
   for (int i = 0; i < np; ++i)
-    for (int k = 0; k < 4 * nfp; ++k) put(2 * TC_BV_BYTES, tc_lcol(i), k, TC_KL, rm.LIFT[size_t(i) * 4 * nfp + k]);
+    for (int k = 0; k < 4 * nfp; ++k) put(2 * TC_BV_BYTES, i, k, TC_KL, rm.LIFT[size_t(i) * 4 * nfp + k]);
   cudaMemcpyToSymbol(gTcB, buf.data(), buf.size() * 4);
 }
