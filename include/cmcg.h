@@ -341,7 +341,7 @@ int cmcg_solve_multifreq(cmcg_handle* h, int nharm, const int* harmonics, const 
  * double[nt][6][Np] host arrays. */
 int cmcg_inner(cmcg_handle* h, const double* u, const double* v, double* out);
 
-/* Largest nt accepted by cmcg_inner_noalloc (128 tetrahedra per block x 8192 blocks). */
+/* Largest nt accepted by cmcg_inner_noalloc. */
 #define CMCG_NOALLOC_MAX_TETS 1048576
 
 /* The paper has no counterpart: this is cmcg_inner without a handle and
@@ -359,10 +359,9 @@ int cmcg_inner(cmcg_handle* h, const double* u, const double* v, double* out);
  * current device and returns once its two kernels are launched; *out is valid
  * when the stream reaches that point.  It reduces through a 64 KiB static
  * device array that every GPU loading the library holds until the process
- * exits.  The first call on a device does a one-time set-up (uploads the mass
- * matrices, looks up the array's device address); make that first call before
- * any stream capture.  All calls share the array: calls that overlap on the
- * GPU race. */
+ * exits.  The first call on a device does a one-time set-up (looks up the
+ * array's device address); make that first call before any stream capture.
+ * All calls share the array: calls that overlap on the GPU race. */
 int cmcg_inner_noalloc(int order, int64_t nt, const double* u, const double* v, const double* w, double* out,
                        void* stream);
 
