@@ -295,7 +295,8 @@ void upload_constants<CMCG_Q>(const RefMats& rm) {
   cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributePreferredSharedMemoryCarveout,
                        int(cudaSharedmemCarveoutMaxShared));  // two P3 CTAs per SM need 2 x 113 KB
   tc_upload_reference(rm);
-  std::vector<float> Df, Lf(rm.LIFT.begin(), rm.LIFT.end());
+  std::vector<float> Df, Lf(rm.LIFT.size());  // LIFT: [node][face node]
+  for (size_t k = 0; k < Lf.size(); ++k) Lf[(k % (4 * NFPQ)) * NPQ + k / (4 * NFPQ)] = float(rm.LIFT[k]);
   for (const std::vector<double>* D : {&rm.Dr, &rm.Ds, &rm.Dt}) Df.insert(Df.end(), D->begin(), D->end());
   if (CMCG_Q == 3) cudaMemcpyToSymbol(cD, Df.data(), sizeof(float) * Df.size());
   cudaMemcpyToSymbol(cL, Lf.data(), sizeof(float) * Lf.size());
