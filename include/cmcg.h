@@ -131,9 +131,9 @@ typedef struct cmcg_mesh {
  *   stage_variant:    0 = time the stage-kernel forms on this mesh at
  *                     creation and keep the fastest; k > 0 forces form k - 1.
  *                     FP32: 0, 1, 2 = two threads per tetrahedron (E / H),
- *                     one warp per 16 tetrahedra, with at least 3, 4, 6
- *                     resident 128-thread blocks per SM; 3, 4 = two warps
- *                     per 16 tetrahedra with at least 3, 4; 5 = four warps;
+ *                     one warp per 16 tetrahedra, with at least 12, 16, 24
+ *                     resident warps per SM; 3, 4 = two warps per 16
+ *                     tetrahedra with at least 12, 16; 5 = four warps;
  *                     6 = the volume and lift contractions on the tensor
  *                     cores (tcgen05, three TF32 products per FP32 product,
  *                     FP32 accumulation).  Forms 0 to 5 give the same bits;

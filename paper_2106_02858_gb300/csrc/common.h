@@ -173,8 +173,8 @@ struct StageArgs {
 
 // Kernel launchers, one translation unit per order.
 // form: stage-kernel form.  FP32: 0, 1, 2 = one warp per half tile (two threads per
-// tetrahedron) with at least 3, 4, 6 resident 128-thread blocks per SM; 3, 4 = two warps
-// per half tile with at least 3, 4 blocks; 5 = four warps per half tile; 6 = tensor-core
+// tetrahedron) with at least 12, 16, 24 resident warps per SM; 3, 4 = two warps
+// per half tile with at least 12, 16; 5 = four warps per half tile; 6 = tensor-core
 // contractions (tcgen05, 3xTF32).  FP64: 0, 1, 2 = one, two, four warps per half tile.
 // pdl: launch with programmatic stream serialisation (the stage overlaps the
 // previous stage's tail).

@@ -268,7 +268,7 @@ void launch_stage<CMCG_Q, float>(const StageArgs<float>& a, cudaStream_t s, int 
     case STAGE_FORM_TC:
       launch_k(dg_stage_tc<TC_MINB>, unsigned((a.nti + TC_TETS - 1) / TC_TETS), TC_THREADS, tc_smem(), s, pdl, a);
       break;
-    default: launch_form<float, 1, 4, 3>(a, s, pdl); break;
+    default: launch_form<float, 1, 2, 6>(a, s, pdl); break;
   }
 }
 template <>
@@ -283,7 +283,7 @@ void launch_stage<CMCG_Q, double>(const StageArgs<double>& a, cudaStream_t s, in
 template <>
 void upload_constants<CMCG_Q>(const RefMats& rm) {
   // allow dynamic shared memory beyond the 48 KiB default
-  allow_smem<float, 1, 4, 3>();
+  allow_smem<float, 1, 2, 6>();
   allow_smem<float, 1, 4, 4>();
   allow_smem<float, 1, 4, 6>();
   allow_smem<float, 2, 4, 3>();

@@ -6,11 +6,20 @@
 // others are immediate operands.  At P3 they, and the lift at every order, are constant-bank
 // operands.  Each output value's sums run in a fixed order (derivatives over j, the lift over faces
 // and face nodes), whatever the split.
+//
+// Issue slots and the latency of a half tile's first loads bound it, not the FP32 pipe (7 of 15.5 us at
+// 82,944 P2 tetrahedra) or the bytes (11 us).  So two values go through one packed instruction
+// wherever two neighbours have the same factor or the same place in a sum; the pipe's rate is that of
+// single ones, but warp instructions and time of that stage were 13.2 M and 19.2 us with single ones,
+// 11.1 M and 16.5 us with the lift packed, 9.1 M and 15.5 us with the fluxes and, at P2, the volume
+// sums too.  Twelve warps of 168 registers per SM, in blocks of two (48,000 tetrahedra: 9.7 us in blocks
+// of four, 9.5 of two; one-warp blocks 12.9); sixteen of 128 registers take 10.6 us there.
 __constant__ float cD[CMCG_Q == 3 ? 3 * NPQ * NPQ : 1];
 __constant__ __align__(8) float cL[4 * NFPQ * NPQ];  // [face node][node]
 
-// (x.lo, x.hi) = (a.lo b.lo + c.lo, a.hi b.hi + c.hi), each rounded once as by fmaf.
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+// Multiply-add and product of two values at once, each rounded once as by fmaf and *; the same names
+// for one value.
+__device__ __forceinline__ float2 vfma(float2 a, float2 b, float2 c) {
   float2 d;
   asm("{\n.reg .b64 x, y, z, r;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %5};\nmov.b64 z, {%6, %7};\n"
       "fma.rn.f32x2 r, x, y, z;\nmov.b64 {%0, %1}, r;\n}\n"
@@ -18,9 +27,23 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
       : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
   return d;
 }
+__device__ __forceinline__ float2 vmul(float2 a, float2 b) {
+  float2 d;
+  asm("{\n.reg .b64 x, y, r;\nmov.b64 x, {%2, %3};\nmov.b64 y, {%4, %5};\n"
+      "mul.rn.f32x2 r, x, y;\nmov.b64 {%0, %1}, r;\n}\n"
+      : "=f"(d.x), "=f"(d.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return d;
+}
+__device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ float vmul(float a, float b) { return __fmul_rn(a, b); }
+template <typename T>
+__device__ __forceinline__ T splat(float a) {
+  if constexpr (sizeof(T) == 8) return {a, a};
+  else return a;
+}
 // phi[n - I0] += L[n][k] fl for the nodes n = I0 .. I0 + NN - 1 and face node k, two nodes per
-// instruction: the pipe's rate is the same as for single ones, but the kernel is bound by issue slots
-// and latency (82,944 P2 tetrahedra: 13.2 M and 11.1 M warp instructions, 19.2 and 16.5 us).
+// instruction.
 template <int I0, int NN>
 __device__ __forceinline__ void nodal_lift(float (&phi)[NN], float fl, int k) {
   const float* L = cL + k * NPQ;
@@ -28,7 +51,7 @@ __device__ __forceinline__ void nodal_lift(float (&phi)[NN], float fl, int k) {
   for (int n = I0 & ~1; n < I0 + NN; n += 2) {
     if (n >= I0 && n + 1 < I0 + NN) {
       const float2 w = *reinterpret_cast<const float2*>(L + n);
-      const float2 r = fma2(w, {fl, fl}, {phi[n - I0], phi[n + 1 - I0]});
+      const float2 r = vfma(w, splat<float2>(fl), {phi[n - I0], phi[n + 1 - I0]});
       phi[n - I0] = r.x;
       phi[n + 1 - I0] = r.y;
     } else {
@@ -67,21 +90,50 @@ constexpr NodalD make_nodal_d() {
   return t;
 }
 
+// The flux of a face at one or two of its nodes: jumps X and the partner's Y, normal n, (k1, k2).
+template <typename T>
+__device__ __forceinline__ void flux_nodes(T (&fl)[3], const T (&X)[3], const T (&Y)[3], float n0, float n1, float n2,
+                                           float k1, float k2) {
+  const float n[3] = {n0, n1, n2};
+  const T nY = vfma(splat<T>(n2), Y[2], vfma(splat<T>(n0), Y[0], vmul(splat<T>(n1), Y[1])));
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int a = (c + 1) % 3, b = (c + 2) % 3;
+    const T nX = vfma(splat<T>(n[a]), X[b], vmul(splat<T>(-n[b]), X[a]));  // (n x X)_c
+    const T tY = vfma(splat<T>(-n[c]), nY, Y[c]);                         // (Y - n (n.Y))_c
+    fl[c] = vfma(splat<T>(k1), nX, vmul(splat<T>(k2), tY));
+  }
+}
 // The flux of face f at its nodes: normal n, (k1, k2), trace weight wt, neighbour trace tr.
 __device__ __forceinline__ void nodal_flux(float (&fl)[3][NFPQ], const float (&tr)[3][NFPQ], const float (&v)[3][NPQ],
                                            float n0, float n1, float n2, float k1, float k2, float wt, int f) {
   constexpr FaceTab FM = make_fmask(CMCG_Q);
 #pragma unroll
-  for (int jf = 0; jf < NFPQ; ++jf) {
-    float X[3], Y[3];
+  for (int jf = 0; jf < NFPQ; jf += 2) {
+    if (jf + 1 < NFPQ) {
+      float2 X[3], Y[3], F[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) X[c] = fmaf(wt, tr[c][jf], -v[c][FM.v[f][jf]]);
+      for (int c = 0; c < 3; ++c)
+        X[c] = {fmaf(wt, tr[c][jf], -v[c][FM.v[f][jf]]), fmaf(wt, tr[c][jf + 1], -v[c][FM.v[f][jf + 1]])};
 #pragma unroll
-    for (int c = 0; c < 3; ++c) Y[c] = __shfl_xor_sync(0xffffffffu, X[c], 1);
-    const float nY = n0 * Y[0] + n1 * Y[1] + n2 * Y[2];
-    fl[0][jf] = k1 * (n1 * X[2] - n2 * X[1]) + k2 * (Y[0] - n0 * nY);
-    fl[1][jf] = k1 * (n2 * X[0] - n0 * X[2]) + k2 * (Y[1] - n1 * nY);
-    fl[2][jf] = k1 * (n0 * X[1] - n1 * X[0]) + k2 * (Y[2] - n2 * nY);
+      for (int c = 0; c < 3; ++c)
+        Y[c] = {__shfl_xor_sync(0xffffffffu, X[c].x, 1), __shfl_xor_sync(0xffffffffu, X[c].y, 1)};
+      flux_nodes<float2>(F, X, Y, n0, n1, n2, k1, k2);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        fl[c][jf] = F[c].x;
+        fl[c][jf + 1] = F[c].y;
+      }
+    } else {
+      float X[3], Y[3], F[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) X[c] = fmaf(wt, tr[c][jf], -v[c][FM.v[f][jf]]);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) Y[c] = __shfl_xor_sync(0xffffffffu, X[c], 1);
+      flux_nodes<float>(F, X, Y, n0, n1, n2, k1, k2);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) fl[c][jf] = F[c];
+    }
   }
 }
 
@@ -148,24 +200,52 @@ __device__ __forceinline__ void nodal_part(const StageArgs<float>& a, int64_t ht
 #pragma unroll
   for (int ii = 0; ii < NN; ++ii) {
     const int i = I0 + ii;
-    float d[3][3];  // [direction][component]
+    if constexpr (CMCG_Q == 1) {  // sums of two terms: nothing to pack (4,374 tetrahedra: 2.7 us packed, 2.45 so)
+      float d[3][3];  // [direction][component]
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      bool first = true;
+      for (int b = 0; b < 3; ++b) {
+        bool first = true;
 #pragma unroll
-      for (int j = 0; j < NP; ++j) {
-        if (CMCG_Q < 3 && D.d[b][i][j] == 0.0f) continue;
-        const float w = CMCG_Q < 3 ? D.d[b][i][j] : cD[(b * NP + i) * NP + j];
+        for (int j = 0; j < NP; ++j) {
+          if (D.d[b][i][j] == 0.0f) continue;
 #pragma unroll
-        for (int c = 0; c < 3; ++c) d[b][c] = first ? w * v[c][j] : fmaf(w, v[c][j], d[b][c]);
-        first = false;
+          for (int c = 0; c < 3; ++c) d[b][c] = first ? D.d[b][i][j] * v[c][j] : fmaf(D.d[b][i][j], v[c][j], d[b][c]);
+          first = false;
+        }
       }
+      // d/dx_ax of component c = sum_b G[b][ax] d[b][c]
+      auto dx = [&](int ax, int c) { return G[0 * 3 + ax] * d[0][c] + G[1 * 3 + ax] * d[1][c] + G[2 * 3 + ax] * d[2][c]; };
+      phi[0][ii] = sv * (dx(1, 2) - dx(2, 1));
+      phi[1][ii] = sv * (dx(2, 0) - dx(0, 2));
+      phi[2][ii] = sv * (dx(0, 1) - dx(1, 0));
+    } else {
+      float2 d10[3];  // d/db of components (1, 0)
+      float d2[3];    // of component 2
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        bool first = true;
+#pragma unroll
+        for (int j = 0; j < NP; ++j) {
+          if (CMCG_Q < 3 && D.d[b][i][j] == 0.0f) continue;
+          const float w = CMCG_Q < 3 ? D.d[b][i][j] : cD[(b * NP + i) * NP + j];
+          const float2 v10 = {v[1][j], v[0][j]}, ww = {w, w};
+          d10[b] = first ? vmul(ww, v10) : vfma(ww, v10, d10[b]);
+          d2[b] = first ? vmul(w, v[2][j]) : vfma(w, v[2][j], d2[b]);
+          first = false;
+        }
+      }
+      // d/dx_ax of component c = sum_b G[b][ax] d[b][c], two at a time
+      auto sum = [&](float2 g0, float2 e0, float2 g1, float2 e1, float2 g2, float2 e2) {
+        return vfma(g2, e2, vfma(g0, e0, vmul(g1, e1)));
+      };
+      const float2 z = sum(splat<float2>(G[2]), d10[0], splat<float2>(G[5]), d10[1], splat<float2>(G[8]), d10[2]);
+      const float2 xy = sum({G[0], G[1]}, d10[0], {G[3], G[4]}, d10[1], {G[6], G[7]}, d10[2]);
+      const float2 xy2 = sum({G[0], G[1]}, splat<float2>(d2[0]), {G[3], G[4]}, splat<float2>(d2[1]), {G[6], G[7]},
+                             splat<float2>(d2[2]));
+      phi[0][ii] = sv * (xy2.y - z.x);
+      phi[1][ii] = sv * (z.y - xy2.x);
+      phi[2][ii] = sv * (xy.x - xy.y);
     }
-    // d/dx_ax of component c = sum_b G[b][ax] d[b][c]
-    auto dx = [&](int ax, int c) { return G[0 * 3 + ax] * d[0][c] + G[1 * 3 + ax] * d[1][c] + G[2 * 3 + ax] * d[2][c]; };
-    phi[0][ii] = sv * (dx(1, 2) - dx(2, 1));
-    phi[1][ii] = sv * (dx(2, 0) - dx(0, 2));
-    phi[2][ii] = sv * (dx(0, 1) - dx(1, 0));
   }
   float bv[3][NN], jv[3][NN];
   float* mine = gsm + GEO32 + l;  // this warp's fluxes (SPLIT > 1)
