@@ -162,6 +162,13 @@ struct cmcg_handle {
   std::map<std::tuple<int, const void*, bool>, cudaGraphExec_t> graph_exec;
   int form = 0;      // stage-kernel form (see launch_stage)
   bool pdl = false;  // stages launched with programmatic stream serialisation
+  // Stages alternate in direction, so that each begins with what the last one has left in L2, from
+  // where the fields they touch and the geometry take more than 3/5 of it.  Microseconds per stage in
+  // one direction and in both: P2 FP32 75 MB 15.5 and 15.7, 84 MB 18.1 and 17.9, 106 MB 26.3 and 22.2,
+  // 146 MB 35.0 and 29.8, 345 MB 74.6 and 68.9; P1 62 MB 11.2 and 11.4, 92 MB 18.2 and 16.8, 154 MB
+  // 34.4 and 28.2; P3 78 MB 32.9 and 33.4, 90 MB 40.6 and 38.0; FP64 within 1% at every size.
+  bool alternate = false;
+  int32_t flip = 0;  // direction of the last launched stage
   double tune_us[10];     // [0..6] per form, [7] the chosen form with overlapped launches, [8..9] unused
   int32_t* err = nullptr;       // device status word of the stage kernels' bounded waits
   int32_t* err_host = nullptr;  // pinned
@@ -350,6 +357,7 @@ void stage(cmcg_handle* h, StageArgs<R>& a, cudaStream_t st) {
   a.err = h->err;
   a.sigma = h->has_sigma ? 1 : 0;
   a.tprob = h->tprob;
+  a.flip = h->alternate ? h->flip ^= 1 : 0;
   if (h->q == 1) launch_stage<1, R>(a, st, h->form, h->pdl);
   else if (h->q == 2) launch_stage<2, R>(a, st, h->form, h->pdl);
   else launch_stage<3, R>(a, st, h->form, h->pdl);
@@ -1322,6 +1330,9 @@ int create_impl(int nprob, const cmcg_problem* probs, const cmcg_options* opt_in
     return fail(CMCG_ERR_OUT_OF_MEMORY);
   if (cudaMemset(h->err, 0, sizeof(int32_t)) != cudaSuccess)
     return fail(CMCG_ERR_CUDA);
+  int l2 = 0;
+  if (cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, opt.device) != cudaSuccess) return fail(CMCG_ERR_CUDA);
+  h->alternate = 5 * (3 * vb + geo.size() * h->rsize + nbr.size() * sizeof(nbr[0])) > 3 * size_t(l2);
   rc = h->prec == CMCG_FP32 ? build_tables<float>(h) : build_tables<double>(h);
   if (rc) return fail(rc);
   if (opt.stage_variant > 0) {

@@ -199,7 +199,7 @@ template <typename R, int SPLIT, int WARPS, int MINB>
 __global__ void __launch_bounds__(32 * WARPS, MINB) dg_stage_kernel(const StageArgs<R> a) {
   grid_dep_launch();
   const int warp = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const int64_t ht = (int64_t(blockIdx.x) * WARPS + warp) / SPLIT;
+  const int64_t ht = (int64_t(a.flip ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * WARPS + warp) / SPLIT;
   if (ht * HTILE >= a.nti) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   R* xs = reinterpret_cast<R*>(smem_raw);

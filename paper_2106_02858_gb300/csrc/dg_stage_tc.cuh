@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) dg_stage_tc(const StageArgs<
   constexpr int KM = (TC_KL / 8 + 1) / 2 * 8;  // lift operand columns written by warpgroup 0, the rest by 1
   grid_dep_launch();
   const int tid = threadIdx.x, wg = tid >> 7, row = tid & 127, warp = row >> 5, l = tid & 31, half = l & 1;
-  const int64_t ht = int64_t(blockIdx.x) * (TC_ROWS / 32) + warp;
+  const int64_t ht = int64_t(a.flip ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * (TC_ROWS / 32) + warp;
   const bool in_range = ht * HTILE < a.nti;  // warp-uniform
 
   // Batches 0, 1: volume of own components 0 and 1, then 2; 2, 3: lift of output components 0 and 1, then 2.
