@@ -528,14 +528,16 @@ void sweep_source(cmcg_handle* h, bool with_source, bool filter, const int32_t* 
   prof_end(h, pe);
 }
 
-// Times the stage-kernel forms [first, first + nforms) on this batch with a nested source-free stage
-// on zero fields (3 warm-up + 12 timed launches each), with overlapped and with plain launches unless
-// the caller asks for one of them, and keeps the fastest pair; tune_us[f] is the faster time of form f
-// (-1: not timed or rejected by the device), tune_us[7] that of the chosen form overlapped.  Both are
-// timed for every form, since either can lose: launches that wait for each other end on a 2 us raster
-// that hides what tells small forms apart, and blocks launched early take the registers that the
-// running stage's last blocks need (P3 FP64, 2,058 tetrahedra: 39.9 us overlapped, 26.8 plain).  The forms of one range give
-// the same bits.
+// Times the stage-kernel forms [first, first + nforms) on this batch with chains of twelve source-free
+// stages on zero fields, launched as the sweeps launch them (as a graph, if the handle uses graphs, each
+// stage reading what the last one wrote: stages that all read the same field showed 3.5 us for forms
+// that take 4.0 and 3.2 in the sweeps of 13,182 P1 tetrahedra), with overlapped and with plain launches
+// unless the caller asks for one of them, and keeps the fastest pair; tune_us[f] is the faster time of
+// form f (-1: not timed or rejected by the device), tune_us[7] that of the chosen form overlapped.  Both
+// are timed for every form, since either can lose: launches that wait for each other end on a 2 us
+// raster, and blocks launched early take the registers that the running stage's last blocks need (P3
+// FP64, 2,058 tetrahedra: 39.9 us overlapped, 26.8 plain).  The forms of one range give the same bits.
+constexpr int TUNE_KIND = 64;  // sweep kinds from here on: autotune's chains
 template <typename R>
 int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
   for (double& x : h->tune_us) x = -1;
@@ -543,33 +545,40 @@ int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
   CK(cudaEventCreate(&e0));
   CK(cudaEventCreate(&e1));
   CK(cudaMemsetAsync(h->Uw, 0, h->nvec * h->rsize, h->stream));
+  CK(cudaMemsetAsync(h->vA, 0, h->nvec * h->rsize, h->stream));
   CK(cudaMemsetAsync(h->vB, 0, h->nvec * h->rsize, h->stream));
   const int64_t launches0 = h->launches;
+  auto chain = [&](cudaStream_t st, int n) {
+    for (int k = 0; k < n; ++k) {
+      StageArgs<R> a = blank<R>();
+      a.vin = (const R*)(k & 1 ? h->vA : h->vB);
+      a.base = (const R*)h->Uw;
+      a.out = (R*)(k & 1 ? h->vB : h->vA);
+      a.coef = tab<R>(h->tab_free, 0, h->nprob);
+      stage<R>(h, a, st);
+    }
+  };
   auto time_one = [&](double* us) -> int {
-    auto run = [&](int n) {
-      for (int k = 0; k < n; ++k) {
-        StageArgs<R> a = blank<R>();
-        a.vin = (const R*)h->Uw;
-        a.base = (const R*)h->vB;
-        a.out = (R*)h->vA;
-        a.coef = tab<R>(h->tab_free, 0, h->nprob);
-        stage<R>(h, a);
-      }
-    };
-    run(1);
+    constexpr int N = 12;
+    chain(h->stream, 1);
     if (cudaGetLastError() != cudaSuccess) {  // launch rejected (configuration): form unavailable
       *us = -1;
       return CMCG_OK;
     }
-    run(2);
+    auto run = [&] {
+      run_sweep(h, std::make_tuple(TUNE_KIND + 2 * h->form + int(h->pdl), (const void*)nullptr, false), N,
+                [&](cudaStream_t st) { chain(st, N); });
+    };
+    run();
     CK(cudaEventRecord(e0, h->stream));
-    run(12);
+    run();
+    run();
     CK(cudaEventRecord(e1, h->stream));
     CK(cudaEventSynchronize(e1));
     CK(cudaGetLastError());
     float ms = 0;
     CK(cudaEventElapsedTime(&ms, e0, e1));
-    *us = 1e3 * ms / 12;
+    *us = 1e3 * ms / (2 * N);
     return CMCG_OK;
   };
   double best = 1e300, over = -1;
@@ -596,6 +605,14 @@ int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
   h->form = bestf;
   h->pdl = bestp;
   h->tune_us[7] = over;
+  for (auto it = h->graph_exec.begin(); it != h->graph_exec.end();) {  // the chains' graphs
+    if (std::get<0>(it->first) >= TUNE_KIND) {
+      cudaGraphExecDestroy(it->second);
+      it = h->graph_exec.erase(it);
+    } else {
+      ++it;
+    }
+  }
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   h->launches = launches0;
@@ -1335,6 +1352,12 @@ int create_impl(int nprob, const cmcg_problem* probs, const cmcg_options* opt_in
   h->alternate = 5 * (3 * vb + geo.size() * h->rsize + nbr.size() * sizeof(nbr[0])) > 3 * size_t(l2);
   rc = h->prec == CMCG_FP32 ? build_tables<float>(h) : build_tables<double>(h);
   if (rc) return fail(rc);
+  h->graphs = opt.launch_graphs != 2;
+  if (h->graphs && cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
+    cudaGetLastError();
+    h->cap_stream = nullptr;
+    h->graphs = false;
+  }
   if (opt.stage_variant > 0) {
     const int nf = h->prec == CMCG_FP32 ? STAGE_FORMS_F32 : STAGE_FORMS_F64;
     if (opt.stage_variant > nf) return fail(CMCG_ERR_INVALID_ARG);
@@ -1348,12 +1371,6 @@ int create_impl(int nprob, const cmcg_problem* probs, const cmcg_options* opt_in
     else if (h->q == 3) rc = autotune<float>(h, STAGE_FORM_TC, 1, opt.stage_overlap);
     else rc = autotune<float>(h, 0, STAGE_FORM_TC, opt.stage_overlap);
     if (rc) return fail(rc);
-  }
-  h->graphs = opt.launch_graphs != 2;
-  if (h->graphs && cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess) {
-    cudaGetLastError();
-    h->cap_stream = nullptr;
-    h->graphs = false;
   }
   h->launches = 0;
   *out = h;
