@@ -220,8 +220,6 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) dg_stage_kernel(const StageA
 
 #include "dg_stage_tc.cuh"
 
-}  // namespace
-
 // Dynamic shared memory: every warp's partial sums (FP64, SPLIT > 1), or geometry and base rows or
 // fluxes (FP32).
 template <typename R, int SPLIT, int WARPS>
@@ -256,6 +254,8 @@ void allow_smem() {
   cudaFuncSetAttribute(dg_stage_kernel<R, SPLIT, WARPS, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        int(stage_smem<R, SPLIT, WARPS>()));
 }
+
+}  // namespace
 
 template <>
 void launch_stage<CMCG_Q, float>(const StageArgs<float>& a, cudaStream_t s, int form, bool pdl) {
