@@ -358,9 +358,9 @@ void stage(cmcg_handle* h, StageArgs<R>& a, cudaStream_t st) {
   a.sigma = h->has_sigma ? 1 : 0;
   a.tprob = h->tprob;
   a.flip = h->alternate ? h->flip ^= 1 : 0;
-  if (h->q == 1) launch_stage<1, R>(a, st, h->form, h->pdl);
-  else if (h->q == 2) launch_stage<2, R>(a, st, h->form, h->pdl);
-  else launch_stage<3, R>(a, st, h->form, h->pdl);
+  if (h->q == 1) launch_stage<1, R>(a, st, h->form, h->pdl, h->nsm);
+  else if (h->q == 2) launch_stage<2, R>(a, st, h->form, h->pdl, h->nsm);
+  else launch_stage<3, R>(a, st, h->form, h->pdl, h->nsm);
 }
 template <typename R>
 void stage(cmcg_handle* h, StageArgs<R>& a) {
@@ -572,13 +572,12 @@ int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
     run();
     CK(cudaEventRecord(e0, h->stream));
     run();
-    run();
     CK(cudaEventRecord(e1, h->stream));
     CK(cudaEventSynchronize(e1));
     CK(cudaGetLastError());
     float ms = 0;
     CK(cudaEventElapsedTime(&ms, e0, e1));
-    *us = 1e3 * ms / (2 * N);
+    *us = 1e3 * ms / N;
     return CMCG_OK;
   };
   double best = 1e300, over = -1;

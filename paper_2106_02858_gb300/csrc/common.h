@@ -178,12 +178,12 @@ struct StageArgs {
 // per half tile with at least 12, 16; 5 = four warps per half tile; 6 = tensor-core
 // contractions (tcgen05, 3xTF32).  FP64: 0, 1, 2 = one, two, four warps per half tile.
 // pdl: launch with programmatic stream serialisation (the stage overlaps the
-// previous stage's tail).
+// previous stage's tail).  nsm: the device's SMs.
 constexpr int STAGE_FORMS_F32 = 7;
 constexpr int STAGE_FORM_TC = 6;
 constexpr int STAGE_FORMS_F64 = 3;
 template <int Q, typename R>
-void launch_stage(const StageArgs<R>& a, cudaStream_t s, int form, bool pdl);
+void launch_stage(const StageArgs<R>& a, cudaStream_t s, int form, bool pdl, int nsm);
 template <int Q>
 void upload_constants(const RefMats& rm);
 

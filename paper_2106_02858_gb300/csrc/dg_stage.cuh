@@ -227,6 +227,18 @@ constexpr size_t stage_smem() {
   if (sizeof(R) == 8) return SPLIT > 1 ? size_t(WARPS) * 3 * NPQ * 32 * sizeof(R) : 0;
   return size_t(WARPS) * nodal_smem<SPLIT>() * sizeof(R);
 }
+// Shared memory per block such that no SM takes more blocks than an even spread over the SMs gives it.
+// The blocks of a grid that does not fill the chip otherwise start where earlier stages' blocks, running
+// or waiting, have left room, two or three to an SM with other SMs idle.  Whole sweeps without and with
+// it: P1 FP32 4,374 tetrahedra 541 and 380 us, 48,000 2,241 and 1,925; P2 FP32 4,374 2,110 and 1,507;
+// P1 FP64 1,296 1,602 and 778; P3 FP64 2,058 6,667 and 6,530; P3 tensor cores 4,374 3,063 and 2,906; 384 of any
+// the same.  P2 FP32 with two or four warps a half tile loses by it (1,296: 994 and 1,160).
+constexpr size_t SM_SHARED = 228 * 1024, BLOCK_RESERVED = 1024, MAX_DYNAMIC = 128 * 1024;
+inline size_t spread_smem(size_t need, int64_t blocks, int nsm) {
+  const int64_t per_sm = (blocks + nsm - 1) / nsm;
+  const size_t pad = SM_SHARED / size_t(per_sm + 1) / 128 * 128 + 128 - BLOCK_RESERVED;  // per_sm + 1 such blocks don't fit
+  return per_sm < 32 && pad > need && (pad + BLOCK_RESERVED) * size_t(per_sm) <= SM_SHARED ? pad : need;
+}
 template <typename Arg>
 void launch_k(void (*k)(Arg), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s, bool pdl,
               const Arg& a) {
@@ -244,39 +256,42 @@ void launch_k(void (*k)(Arg), unsigned blocks, unsigned threads, size_t smem, cu
 }
 
 template <typename R, int SPLIT, int WARPS, int MINB>
-void launch_form(const StageArgs<R>& a, cudaStream_t s, bool pdl) {
-  const int64_t warps = a.nti / HTILE * SPLIT;
-  launch_k(dg_stage_kernel<R, SPLIT, WARPS, MINB>, unsigned((warps + WARPS - 1) / WARPS), 32 * WARPS,
-           stage_smem<R, SPLIT, WARPS>(), s, pdl, a);
+void launch_form(const StageArgs<R>& a, cudaStream_t s, bool pdl, int nsm) {
+  constexpr bool spread = sizeof(R) == 8 || SPLIT == 1 || CMCG_Q == 1;
+  constexpr size_t need = stage_smem<R, SPLIT, WARPS>();
+  const int64_t warps = a.nti / HTILE * SPLIT, blocks = (warps + WARPS - 1) / WARPS;
+  launch_k(dg_stage_kernel<R, SPLIT, WARPS, MINB>, unsigned(blocks), 32 * WARPS,
+           spread ? spread_smem(need, blocks, nsm) : need, s, pdl, a);
 }
 template <typename R, int SPLIT, int WARPS, int MINB>
 void allow_smem() {
   cudaFuncSetAttribute(dg_stage_kernel<R, SPLIT, WARPS, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                       int(stage_smem<R, SPLIT, WARPS>()));
+                       int(MAX_DYNAMIC));
 }
 
 }  // namespace
 
 template <>
-void launch_stage<CMCG_Q, float>(const StageArgs<float>& a, cudaStream_t s, int form, bool pdl) {
+void launch_stage<CMCG_Q, float>(const StageArgs<float>& a, cudaStream_t s, int form, bool pdl, int nsm) {
   switch (form) {
-    case 1: launch_form<float, 1, 4, 4>(a, s, pdl); break;
-    case 2: launch_form<float, 1, 4, 6>(a, s, pdl); break;
-    case 3: launch_form<float, 2, 4, 3>(a, s, pdl); break;
-    case 4: launch_form<float, 2, 4, 4>(a, s, pdl); break;
-    case 5: launch_form<float, 4, 4, 4>(a, s, pdl); break;
+    case 1: launch_form<float, 1, 4, 4>(a, s, pdl, nsm); break;
+    case 2: launch_form<float, 1, 4, 6>(a, s, pdl, nsm); break;
+    case 3: launch_form<float, 2, 4, 3>(a, s, pdl, nsm); break;
+    case 4: launch_form<float, 2, 4, 4>(a, s, pdl, nsm); break;
+    case 5: launch_form<float, 4, 4, 4>(a, s, pdl, nsm); break;
     case STAGE_FORM_TC:
-      launch_k(dg_stage_tc<TC_MINB>, unsigned((a.nti + TC_TETS - 1) / TC_TETS), TC_THREADS, tc_smem(), s, pdl, a);
+      launch_k(dg_stage_tc<TC_MINB>, unsigned((a.nti + TC_TETS - 1) / TC_TETS), TC_THREADS,
+               spread_smem(tc_smem(), (a.nti + TC_TETS - 1) / TC_TETS, nsm), s, pdl, a);
       break;
-    default: launch_form<float, 1, 2, 6>(a, s, pdl); break;
+    default: launch_form<float, 1, 2, 6>(a, s, pdl, nsm); break;
   }
 }
 template <>
-void launch_stage<CMCG_Q, double>(const StageArgs<double>& a, cudaStream_t s, int form, bool pdl) {
+void launch_stage<CMCG_Q, double>(const StageArgs<double>& a, cudaStream_t s, int form, bool pdl, int nsm) {
   switch (form) {
-    case 1: launch_form<double, 2, 2, 1>(a, s, pdl); break;
-    case 2: launch_form<double, 4, 4, 1>(a, s, pdl); break;
-    default: launch_form<double, 1, 4, 1>(a, s, pdl); break;
+    case 1: launch_form<double, 2, 2, 1>(a, s, pdl, nsm); break;
+    case 2: launch_form<double, 4, 4, 1>(a, s, pdl, nsm); break;
+    default: launch_form<double, 1, 4, 1>(a, s, pdl, nsm); break;
   }
 }
 
@@ -289,9 +304,10 @@ void upload_constants<CMCG_Q>(const RefMats& rm) {
   allow_smem<float, 2, 4, 3>();
   allow_smem<float, 2, 4, 4>();
   allow_smem<float, 4, 4, 4>();
+  allow_smem<double, 1, 4, 1>();
   allow_smem<double, 2, 2, 1>();
   allow_smem<double, 4, 4, 1>();
-  cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(tc_smem()));
+  cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(MAX_DYNAMIC));
   cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributePreferredSharedMemoryCarveout,
                        int(cudaSharedmemCarveoutMaxShared));  // two P3 CTAs per SM need 2 x 113 KB
   tc_upload_reference(rm);
