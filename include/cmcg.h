@@ -141,12 +141,10 @@ typedef struct cmcg_mesh {
  *                     order 3.  FP64: 0, 1, 2 = one, two, four warps per 16
  *                     tetrahedra.  Other k: CMCG_ERR_INVALID_ARG.  Results do not
  *                     depend on it beyond rounding.
- *   stage_overlap:    0 = the faster when the forms are timed (stage_variant
- *                     0; on for a forced form); 1 = on; 2 = off.  On: each
- *                     stage is launched with programmatic stream
- *                     serialisation, so its blocks start and load the mesh
- *                     data while the previous stage finishes.  Results are
- *                     identical.
+ *   stage_overlap:    0 or 1 = on; 2 = off.  On: each stage
+ *                     is launched with programmatic stream serialisation, so
+ *                     its blocks start and load the mesh data while the
+ *                     previous stage finishes.  Results are identical.
  *   launch_graphs:    0 or 1 = each period sweep (its stage launches) is
  *                     captured once as a CUDA graph on a private stream and
  *                     replayed on the handle's stream; 2 = direct launches.

@@ -169,7 +169,7 @@ struct cmcg_handle {
   // 34.4 and 28.2; P3 78 MB 32.9 and 33.4, 90 MB 40.6 and 38.0; FP64 within 1% at every size.
   bool alternate = false;
   int32_t flip = 0;  // direction of the last launched stage
-  double tune_us[10];     // [0..6] per form, [7] the chosen form with overlapped launches, [8..9] unused
+  double tune_us[10];     // [0..6] per form, [7] the chosen form, [8..9] unused
   int32_t* err = nullptr;       // device status word of the stage kernels' bounded waits
   int32_t* err_host = nullptr;  // pinned
   // sweep profiling
@@ -531,12 +531,11 @@ void sweep_source(cmcg_handle* h, bool with_source, bool filter, const int32_t* 
 // Times the stage-kernel forms [first, first + nforms) on this batch with chains of twelve source-free
 // stages on zero fields, launched as the sweeps launch them (as a graph, if the handle uses graphs, each
 // stage reading what the last one wrote: stages that all read the same field showed 3.5 us for forms
-// that take 4.0 and 3.2 in the sweeps of 13,182 P1 tetrahedra), with overlapped and with plain launches
-// unless the caller asks for one of them, and keeps the fastest pair; tune_us[f] is the faster time of
-// form f (-1: not timed or rejected by the device), tune_us[7] that of the chosen form overlapped.  Both
-// are timed for every form, since either can lose: launches that wait for each other end on a 2 us
-// raster, and blocks launched early take the registers that the running stage's last blocks need (P3
-// FP64, 2,058 tetrahedra: 39.9 us overlapped, 26.8 plain).  The forms of one range give the same bits.
+// that take 4.0 and 3.2 in the sweeps of 13,182 P1 tetrahedra), and keeps the fastest; tune_us[f] is the
+// time of form f (-1: not timed or rejected by the device), tune_us[7] that of the chosen form.  Launches
+// overlap unless the caller forbids it: once a grid is spread evenly (spread_smem) plain launches are
+// slower at every size (P1 FP32 384 tetrahedra 174 and 152 us a sweep, 48,000 2,226 and 1,932; P3 FP64
+// 2,058 6,711 and 6,552).  The forms of one range give the same bits.
 constexpr int TUNE_KIND = 64;  // sweep kinds from here on: autotune's chains
 template <typename R>
 int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
@@ -566,7 +565,7 @@ int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
       return CMCG_OK;
     }
     auto run = [&] {
-      run_sweep(h, std::make_tuple(TUNE_KIND + 2 * h->form + int(h->pdl), (const void*)nullptr, false), N,
+      run_sweep(h, std::make_tuple(TUNE_KIND + h->form, (const void*)nullptr, false), N,
                 [&](cudaStream_t st) { chain(st, N); });
     };
     run();
@@ -580,30 +579,22 @@ int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
     *us = 1e3 * ms / N;
     return CMCG_OK;
   };
-  double best = 1e300, over = -1;
+  h->pdl = overlap != 2;
+  double best = 1e300;
   int bestf = first;
-  bool bestp = overlap != 2;
   for (int f = first; f < first + nforms; ++f) {
-    double us[2] = {-1, -1};  // plain, overlapped
-    for (int p = 1; p >= 0; --p) {
-      if (overlap == 1 + p) continue;  // 1: overlapped only; 2: plain only
-      h->form = f;
-      h->pdl = p;
-      int rc = time_one(&us[p]);
-      if (rc) return rc;
-      if (us[p] < 0) continue;
-      if (h->tune_us[f] < 0 || us[p] < h->tune_us[f]) h->tune_us[f] = us[p];
-      if (us[p] < best) {
-        best = us[p];
-        bestf = f;
-        bestp = p;
-      }
+    h->form = f;
+    double us;
+    const int rc = time_one(&us);
+    if (rc) return rc;
+    h->tune_us[f] = us;
+    if (us >= 0 && us < best) {
+      best = us;
+      bestf = f;
     }
-    if (bestf == f) over = us[1];
   }
   h->form = bestf;
-  h->pdl = bestp;
-  h->tune_us[7] = over;
+  h->tune_us[7] = h->tune_us[bestf];
   for (auto it = h->graph_exec.begin(); it != h->graph_exec.end();) {  // the chains' graphs
     if (std::get<0>(it->first) >= TUNE_KIND) {
       cudaGraphExecDestroy(it->second);
