@@ -171,7 +171,11 @@ struct cmcg_handle {
   int32_t flip = 0;  // direction of the last launched stage
   double tune_us[10];     // [0..6] per form, [7] the chosen form, [8..9] unused
   int32_t* err = nullptr;       // device status word of the stage kernels' bounded waits
-  int32_t* err_host = nullptr;  // pinned
+  // Pinned, one allocation: err_host, the coefficient table of a single application, and, if the arrays
+  // of a single application take at most IO_HOST_MAX together, those (see dgtd_apply).
+  int32_t* err_host = nullptr;
+  void* coef_host = nullptr;
+  double* io_host = nullptr;
   // sweep profiling
   bool prof = false;
   struct SweepEv {
@@ -712,6 +716,10 @@ int adjoint_dev(cmcg_handle* h, const double* wT, double* w0) {
   return check_err(h);
 }
 
+// Arrays of one application that go through pinned memory take at most this many bytes (384 P2
+// tetrahedra, 553 kB: 104 us by copies, 91 so; 750, 1,080 kB: 108 and, by copies with one wait, 105).
+constexpr size_t IO_HOST_MAX = 1 << 20;
+// Launches one application; the caller waits for it (check_err) before the next.
 template <typename R>
 int apply_dev(cmcg_handle* h, double t, const double* u, const double* j_re, const double* j_im, int adjoint,
               double* out) {
@@ -723,8 +731,9 @@ int apply_dev(cmcg_handle* h, double t, const double* u, const double* j_re, con
   c.c_out = R(1);
   c.s_cos = R(std::cos(h->P[0].omega * t));
   c.s_sin = R(std::sin(h->P[0].omega * t));
-  const std::vector<StageCoef<R>> cs(size_t(h->nprob), c);  // every part of a sharded handle
-  CK(cudaMemcpy(h->tab_one, cs.data(), sizeof(c) * cs.size(), cudaMemcpyHostToDevice));
+  StageCoef<R>* cs = static_cast<StageCoef<R>*>(h->coef_host);
+  std::fill(cs, cs + h->nprob, c);  // every part of a sharded handle
+  CK(cudaMemcpyAsync(h->tab_one, cs, sizeof(c) * h->nprob, cudaMemcpyHostToDevice, h->stream));
   StageArgs<R> a = blank<R>();
   a.vin = (const R*)h->Uw;
   a.base = (const R*)h->vB;
@@ -743,7 +752,7 @@ int apply_dev(cmcg_handle* h, double t, const double* u, const double* j_re, con
   stage<R>(h, a);
   for (int p = 0; p < nconv(h); ++p) field_to_ext<R>(h, p, h->vA, out);
   CK(cudaGetLastError());
-  return check_err(h);
+  return CMCG_OK;
 }
 
 template <typename R>
@@ -1330,11 +1339,15 @@ int create_impl(int nprob, const cmcg_problem* probs, const cmcg_options* opt_in
             alloc((void**)&h->ext0, extlen) && alloc((void**)&h->ext1, extlen) && alloc((void**)&h->ext2, extlen) &&
             alloc((void**)&h->ext3, extlen);
   if (!ok) return fail(CMCG_ERR_OUT_OF_MEMORY);
+  const size_t coef_bytes = (sizeof(StageCoef<double>) * nprob + 127) / 128 * 128;
+  const size_t io_bytes = (nprob == 1 || h->coupled) && 3 * extlen <= IO_HOST_MAX ? 3 * extlen : 0;
   if (cudaMallocHost((void**)&h->sc_host, sizeof(Scalars) * nprob) != cudaSuccess ||
       cudaMallocHost((void**)&h->pactive_host, sizeof(int32_t) * nprob) != cudaSuccess ||
       cudaMallocHost((void**)&h->used_host, sizeof(int32_t) * nprob) != cudaSuccess ||
-      cudaMallocHost((void**)&h->err_host, sizeof(int32_t)) != cudaSuccess)
+      cudaMallocHost((void**)&h->err_host, 128 + coef_bytes + io_bytes) != cudaSuccess)
     return fail(CMCG_ERR_OUT_OF_MEMORY);
+  h->coef_host = reinterpret_cast<char*>(h->err_host) + 128;
+  if (io_bytes) h->io_host = reinterpret_cast<double*>(static_cast<char*>(h->coef_host) + coef_bytes);
   if (cudaMemset(h->err, 0, sizeof(int32_t)) != cudaSuccess)
     return fail(CMCG_ERR_CUDA);
   int l2 = 0;
@@ -1623,15 +1636,33 @@ int dgtd_apply(cmcg_handle* h, double t, const double* u, const double* j_re, co
   if (!single(h) || !u || !out) return CMCG_ERR_INVALID_ARG;
   if (cudaSetDevice(h->device) != cudaSuccess) return CMCG_ERR_CUDA;
   const size_t n = size_t(ext_nt(h)) * 6 * h->np, nj = size_t(ext_nt(h)) * 3 * h->np;
-  CK(cudaMemcpyAsync(h->ext0, u, n * 8, cudaMemcpyHostToDevice, h->stream));
-  if (j_re) CK(cudaMemcpyAsync(h->ext2, j_re, nj * 8, cudaMemcpyHostToDevice, h->stream));
-  if (j_re && j_im) CK(cudaMemcpyAsync(h->ext3, j_im, nj * 8, cudaMemcpyHostToDevice, h->stream));
-  const double* jr = j_re ? h->ext2 : nullptr;
-  const double* ji = (j_re && j_im) ? h->ext3 : nullptr;
-  int rc = DISPATCH(h, apply_dev<float>(h, t, h->ext0, jr, ji, adjoint, h->ext1),
-                    apply_dev<double>(h, t, h->ext0, jr, ji, adjoint, h->ext1));
-  if (rc) return rc;
-  CK(cudaMemcpyAsync(out, h->ext1, n * 8, cudaMemcpyDeviceToHost, h->stream));
+  // Small arrays go through pinned memory that the conversion kernels read and write themselves: a
+  // call is four kernels, two small copies and one wait, without a copy command per array (162 P2
+  // tetrahedra: 93 us by copies and three waits, 70 so; FP64 142 and 85).  Larger ones are copied.
+  double* du = h->io_host ? h->io_host : h->ext0;
+  double* dj = h->io_host ? du + n : nullptr;
+  double* dout = h->io_host ? dj + 2 * nj : h->ext1;
+  const double* jr = nullptr;
+  const double* ji = nullptr;
+  if (h->io_host) {
+    std::memcpy(du, u, n * 8);
+    if (j_re) jr = static_cast<double*>(std::memcpy(dj, j_re, nj * 8));
+    if (j_re && j_im) ji = static_cast<double*>(std::memcpy(dj + nj, j_im, nj * 8));
+  } else {
+    CK(cudaMemcpyAsync(du, u, n * 8, cudaMemcpyHostToDevice, h->stream));
+    if (j_re) CK(cudaMemcpyAsync(h->ext2, j_re, nj * 8, cudaMemcpyHostToDevice, h->stream));
+    if (j_re && j_im) CK(cudaMemcpyAsync(h->ext3, j_im, nj * 8, cudaMemcpyHostToDevice, h->stream));
+    jr = j_re ? h->ext2 : nullptr;
+    ji = (j_re && j_im) ? h->ext3 : nullptr;
+  }
+  int rc = DISPATCH(h, apply_dev<float>(h, t, du, jr, ji, adjoint, dout), apply_dev<double>(h, t, du, jr, ji, adjoint, dout));
+  const int st = check_err(h);  // waits, whatever was launched
+  if (rc || (rc = st)) return rc;
+  if (h->io_host) {
+    std::memcpy(out, dout, n * 8);
+    return CMCG_OK;
+  }
+  CK(cudaMemcpyAsync(out, dout, n * 8, cudaMemcpyDeviceToHost, h->stream));
   CK(cudaStreamSynchronize(h->stream));
   return CMCG_OK;
 }
