@@ -8,7 +8,7 @@
 // and face nodes), whatever the split.
 //
 // Issue slots and the latency of a half tile's first loads bound it, not the FP32 pipe (7 of 15.5 us at
-// 82,944 P2 tetrahedra) or the bytes (11 us).  So two values go through one packed instruction
+// 81,648 P2 tetrahedra) or the bytes (11 us).  So two values go through one packed instruction
 // wherever two neighbours have the same factor or the same place in a sum; the pipe's rate is that of
 // single ones, but warp instructions and time of that stage were 13.2 M and 19.2 us with single ones,
 // 11.1 M and 16.5 us with the lift packed, 9.1 M and 15.5 us with the fluxes and, at P2, the volume

@@ -46,7 +46,7 @@ static __device__ __align__(256) double g_na_partials[NA_MAX_BLOCKS];
 //                  - 27 (a b' + b a') - 54 (a f' + f a') + 216 f f') + 2 V V' + 3 (V A' + A V')
 //                  + 18 (V F' + F V') + 216 F F' + 54 sum_e e e'
 // 12, 57 and 135 operations where the dense matrix takes 20, 110 and 420: at GB300's FP64 rate (one
-// warp instruction per 64 cycles and SM quarter) they bound the kernel, not the bytes.  82,944 P2
+// warp instruction per 64 cycles and SM quarter) they bound the kernel, not the bytes.  81,648 P2
 // tetrahedra: 131 us with the dense matrix, 68 us so (80 MB of fields; the operations alone 46 us).
 // The error against exact sums is below the dense matrix's, whose entries were themselves rounded.
 struct NaTab {
