@@ -309,7 +309,7 @@ void upload_constants<CMCG_Q>(const RefMats& rm) {
   allow_smem<double, 4, 4, 1>();
   cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(MAX_DYNAMIC));
   cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                       int(cudaSharedmemCarveoutMaxShared));  // two P3 CTAs per SM need 2 x 113 KB
+                       int(cudaSharedmemCarveoutMaxShared));  // two P3 CTAs per SM need 2 x 95 KB
   tc_upload_reference(rm);
   std::vector<float> Df, Lf(rm.LIFT.size());  // LIFT: [node][face node]
   for (size_t k = 0; k < Lf.size(); ++k) Lf[(k % (4 * NFPQ)) * NPQ + k / (4 * NFPQ)] = float(rm.LIFT[k]);
