@@ -537,9 +537,9 @@ void sweep_source(cmcg_handle* h, bool with_source, bool filter, const int32_t* 
 // stage reading what the last one wrote: stages that all read the same field showed 3.5 us for forms
 // that take 4.0 and 3.2 in the sweeps of 13,182 P1 tetrahedra), and keeps the fastest; tune_us[f] is the
 // time of form f (-1: not timed or rejected by the device), tune_us[7] that of the chosen form.  Launches
-// overlap unless the caller forbids it: once a grid is spread evenly (spread_smem) plain launches are
-// slower at every size (P1 FP32 384 tetrahedra 174 and 152 us a sweep, 48,000 2,226 and 1,932; P3 FP64
-// 2,058 6,711 and 6,552).  The forms of one range give the same bits.
+// overlap unless the caller forbids it: plain launches are slower at nearly every size (P1 FP32 384
+// tetrahedra 174 and 152 us a sweep, 48,000 2,226 and 1,932; P3 FP64 2,058 6,711 and 6,552).  The forms
+// of one range give the same bits.
 constexpr int TUNE_KIND = 64;  // sweep kinds from here on: autotune's chains
 template <typename R>
 int autotune(cmcg_handle* h, int first, int nforms, int overlap) {

@@ -61,6 +61,10 @@ __constant__ unsigned long long cNB[4 * 8];
 // writes are visible, it reads only data that no kernel writes (geometry,
 // neighbour codes, coefficient tables, tile problems).
 // Without the launch attribute both are no-ops.
+// The next stage may start its blocks: called after the grid dependency's wait, so that at most one
+// stage waits.  Called first, several stages pile up, and their waiting blocks make running ones double up
+// on some SMs with others idle (sweeps: P2 FP32 1,296 tetrahedra 994 us, 810 so; 2,058 1,378 and
+// 1,015; P1 FP64 1,296 1,602 and 752).
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
@@ -197,7 +201,6 @@ __device__ __forceinline__ void stage_part(const StageArgs<float>& a, int64_t ht
 // registers at 65536 / (32 WARPS MINB)).  The forms are timed per handle (see api.cu).
 template <typename R, int SPLIT, int WARPS, int MINB>
 __global__ void __launch_bounds__(32 * WARPS, MINB) dg_stage_kernel(const StageArgs<R> a) {
-  grid_dep_launch();
   const int warp = threadIdx.x >> 5, l = threadIdx.x & 31;
   const int64_t ht = (int64_t(a.flip ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * WARPS + warp) / SPLIT;
   if (ht * HTILE >= a.nti) return;
@@ -227,17 +230,16 @@ constexpr size_t stage_smem() {
   if (sizeof(R) == 8) return SPLIT > 1 ? size_t(WARPS) * 3 * NPQ * 32 * sizeof(R) : 0;
   return size_t(WARPS) * nodal_smem<SPLIT>() * sizeof(R);
 }
-// Shared memory per block such that no SM takes more blocks than an even spread over the SMs gives it.
-// The blocks of a grid that does not fill the chip otherwise start where earlier stages' blocks, running
-// or waiting, have left room, two or three to an SM with other SMs idle.  Whole sweeps without and with
-// it: P1 FP32 4,374 tetrahedra 541 and 380 us, 48,000 2,241 and 1,925; P2 FP32 4,374 2,110 and 1,507;
-// P1 FP64 1,296 1,602 and 778; P3 FP64 2,058 6,667 and 6,530; P3 tensor cores 4,374 3,063 and 2,906; 384 of any
-// the same.  P2 FP32 with two or four warps a half tile loses by it (1,296: 994 and 1,160).
+// Shared memory per block such that no SM takes more blocks than an even spread over the SMs gives it,
+// for grids of more blocks than SMs (P1 FP32 24,576 tetrahedra 1,190 us a sweep without it, 1,040 so; 48,000
+// 2,121 and 1,889).  Smaller grids are left alone: a whole SM to a block keeps other handles' kernels
+// out (four handles of 4,374 P1 tetrahedra on four streams 1.29 ms so, 0.83 without).  P2 FP32 with two or
+// four warps a half tile loses by it (1,296 tetrahedra: 994 and 1,160 us).
 constexpr size_t SM_SHARED = 228 * 1024, BLOCK_RESERVED = 1024, MAX_DYNAMIC = 128 * 1024;
 inline size_t spread_smem(size_t need, int64_t blocks, int nsm) {
   const int64_t per_sm = (blocks + nsm - 1) / nsm;
   const size_t pad = SM_SHARED / size_t(per_sm + 1) / 128 * 128 + 128 - BLOCK_RESERVED;  // per_sm + 1 such blocks don't fit
-  return per_sm < 32 && pad > need && (pad + BLOCK_RESERVED) * size_t(per_sm) <= SM_SHARED ? pad : need;
+  return per_sm > 1 && per_sm < 32 && pad > need && (pad + BLOCK_RESERVED) * size_t(per_sm) <= SM_SHARED ? pad : need;
 }
 template <typename Arg>
 void launch_k(void (*k)(Arg), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s, bool pdl,

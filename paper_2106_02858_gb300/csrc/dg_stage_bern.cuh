@@ -157,6 +157,7 @@ __device__ __forceinline__ void bern_part(const StageArgs<double>& a, int64_t ht
   const double sigma = a.sigma ? a.geo[ht * GEO64 + (GEO_S64 * 16 + GEO_SIGMA * 32) + l] : double(0);
 
   grid_dep_wait();
+  grid_dep_launch();
   if (a.pactive && !a.pactive[prob]) return;  // CG converged for this problem (written by the CG kernels)
   const int64_t own = ht * HS + l;  // the thread's field; its output is the partner's, own ^ 1
   // Traces run one face ahead of their use.

@@ -169,6 +169,7 @@ __device__ __forceinline__ void nodal_part(const StageArgs<float>& a, int64_t ht
   for (int ff = 0; ff < NF; ++ff) nb[ff] = find_neighbour(a, ht, l, F0 + ff);
 
   grid_dep_wait();
+  grid_dep_launch();
   if (a.pactive && !a.pactive[prob]) {  // CG converged for this problem (written by the CG kernels)
     cp_async_wait<0>();
     return;

@@ -231,7 +231,6 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) dg_stage_tc(const StageArgs<
   constexpr int NP = NPQ, NFP = NFPQ;
   constexpr FaceTab FM = make_fmask(CMCG_Q);
   constexpr int KM = (TC_KL / 8 + 1) / 2 * 8;  // lift operand columns written by warpgroup 0, the rest by 1
-  grid_dep_launch();
   const int tid = threadIdx.x, wg = tid >> 7, row = tid & 127, warp = row >> 5, l = tid & 31, half = l & 1;
   const int64_t ht = int64_t(a.flip ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * (TC_ROWS / 32) + warp;
   const bool in_range = ht * HTILE < a.nti;  // warp-uniform
@@ -341,6 +340,7 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) dg_stage_tc(const StageArgs<
       asm volatile("" : "+l"(nb[f].at), "+l"(nb[f].nodes));  // looked up before the wait
     }
     grid_dep_wait();
+    grid_dep_launch();
     if (live && a.pactive && !a.pactive[prob]) live = false;  // CG converged (written by the CG kernels)
     if (!cta_or(live)) return;
     // Traces of a face two faces ahead of its fluxes, each face a group of copies.
@@ -428,6 +428,7 @@ __global__ void __launch_bounds__(TC_THREADS, MINB) dg_stage_tc(const StageArgs<
   for (int m = 0; m < 9; ++m) G[m] = gs[m * 16] * sv;  // the material factor of Phi, folded into the chain rule
   const R sigma = a.sigma ? gp[GEO_SIGMA * 32] : R(0);
   grid_dep_wait();
+  grid_dep_launch();
   if (live && a.pactive && !a.pactive[prob]) live = false;
   if (!cta_or(live)) {
     if (tid == 0) mbar_wait(barB, 0);  // the copy lands before the CTA's shared memory is released
