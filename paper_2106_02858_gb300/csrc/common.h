@@ -165,6 +165,7 @@ struct StageArgs {
   int32_t* err;  // device status word: a stage kernel whose bounded wait ran out ORs in 1 (null: not recorded)
   int32_t sigma;  // nonzero: some tetrahedron has a conductivity
   int32_t flip;   // nonzero: the blocks take the tetrahedra from the last to the first
+  int32_t nsm;    // the device's SMs
   // Several harmonics in one sweep (nharm > 0): the source is sum_h hcs[2h] J_re,h - hcs[2h+1] J_im,h
   // with J_h = j + h * jstride (hcs: this launch's cos / sin of the harmonics at the stage time).
   int32_t nharm;

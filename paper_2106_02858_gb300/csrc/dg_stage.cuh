@@ -61,10 +61,12 @@ __constant__ unsigned long long cNB[4 * 8];
 // writes are visible, it reads only data that no kernel writes (geometry,
 // neighbour codes, coefficient tables, tile problems).
 // Without the launch attribute both are no-ops.
-// The next stage may start its blocks: called after the grid dependency's wait, so that at most one
-// stage waits.  Called first, several stages pile up, and their waiting blocks make running ones double up
-// on some SMs with others idle (sweeps: P2 FP32 1,296 tetrahedra 994 us, 810 so; 2,058 1,378 and
-// 1,015; P1 FP64 1,296 1,602 and 752).
+// The next stage may start its blocks: called first by grids of more blocks than SMs (81,648 P2
+// tetrahedra 14.6 ms a sweep when called later, 14.4 so), by smaller ones after the grid dependency's
+// wait, so that at most one stage waits.  There, called first, several stages pile up, and their
+// waiting blocks make running ones double up on some SMs with others idle (sweeps: P2 FP32 1,296
+// tetrahedra 994 us, 810 so; 2,058 1,378 and 1,015; P1 FP64 1,296 1,602 and 752).  The tensor-core
+// stage calls it after the wait at every size (12,288 P3 tetrahedra: within 1% of calling it first).
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
@@ -201,6 +203,7 @@ __device__ __forceinline__ void stage_part(const StageArgs<float>& a, int64_t ht
 // registers at 65536 / (32 WARPS MINB)).  The forms are timed per handle (see api.cu).
 template <typename R, int SPLIT, int WARPS, int MINB>
 __global__ void __launch_bounds__(32 * WARPS, MINB) dg_stage_kernel(const StageArgs<R> a) {
+  if (gridDim.x > unsigned(a.nsm)) grid_dep_launch();
   const int warp = threadIdx.x >> 5, l = threadIdx.x & 31;
   const int64_t ht = (int64_t(a.flip ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * WARPS + warp) / SPLIT;
   if (ht * HTILE >= a.nti) return;
