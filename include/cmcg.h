@@ -139,8 +139,9 @@ typedef struct cmcg_mesh {
  *                     FP32 accumulation).  Forms 0 to 5 give the same bits;
  *                     0 times those at orders 1 and 2 and takes form 6 at
  *                     order 3.  FP64: 0, 1, 2 = one, two, four warps per 16
- *                     tetrahedra.  Other k: CMCG_ERR_INVALID_ARG.  Results do not
- *                     depend on it beyond rounding.
+ *                     tetrahedra, the same bits from each.  Other k:
+ *                     CMCG_ERR_INVALID_ARG.  Results do not depend on it beyond
+ *                     rounding.
  *   stage_overlap:    0 or 1 = on; 2 = off.  On: each stage
  *                     is launched with programmatic stream serialisation, so
  *                     its blocks start and load the mesh data while the

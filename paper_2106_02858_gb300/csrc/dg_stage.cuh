@@ -226,11 +226,11 @@ __global__ void __launch_bounds__(32 * WARPS, MINB) dg_stage_kernel(const StageA
 
 #include "dg_stage_tc.cuh"
 
-// Dynamic shared memory: every warp's partial sums (FP64, SPLIT > 1), or geometry and base rows or
-// fluxes (FP32).
+// Dynamic shared memory: what the warps of a half tile exchange (FP64, SPLIT > 1), or geometry and base
+// rows or fluxes (FP32).
 template <typename R, int SPLIT, int WARPS>
 constexpr size_t stage_smem() {
-  if (sizeof(R) == 8) return SPLIT > 1 ? size_t(WARPS) * 3 * NPQ * 32 * sizeof(R) : 0;
+  if (sizeof(R) == 8) return SPLIT > 1 ? size_t(WARPS / SPLIT) * BERN_SMEM * 32 * sizeof(R) : 0;
   return size_t(WARPS) * nodal_smem<SPLIT>() * sizeof(R);
 }
 // Shared memory per block such that no SM takes more blocks than an even spread over the SMs gives it,
