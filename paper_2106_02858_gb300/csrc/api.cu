@@ -533,17 +533,16 @@ void sweep_source(cmcg_handle* h, bool with_source, bool filter, const int32_t* 
   prof_end(h, pe);
 }
 
-// Times the stage-kernel forms [first, first + nforms) on this batch with chains of twelve source-free
-// stages on zero fields, launched as the sweeps launch them (as a graph, if the handle uses graphs, each
+// Takes the fastest of the stage-kernel forms that choose_form times on this batch, with chains of twelve
+// source-free stages on zero fields, launched as the sweeps launch them (as a graph, if the handle uses graphs, each
 // stage reading what the last one wrote: stages that all read the same field showed 3.5 us for forms
-// that take 4.0 and 3.2 in the sweeps of 13,182 P1 tetrahedra), and keeps the fastest; tune_us[f] is the
+// that take 4.0 and 3.2 in the sweeps of 13,182 P1 tetrahedra); tune_us[f] is the
 // time of form f (-1: not timed or rejected by the device), tune_us[7] that of the chosen form.  Launches
 // overlap unless the caller forbids it: plain launches are slower at nearly every size (P1 FP32 384
-// tetrahedra 174 and 152 us a sweep, 48,000 2,226 and 1,932; P3 FP64 2,058 6,711 and 6,552).  The forms
-// of one range give the same bits.
+// tetrahedra 174 and 152 us a sweep, 48,000 2,226 and 1,932; P3 FP64 2,058 6,711 and 6,552).
 constexpr int TUNE_KIND = 64;  // sweep kinds from here on: autotune's chains
 template <typename R>
-int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
+int autotune(cmcg_handle* h, int overlap) {
   for (double& x : h->tune_us) x = -1;
   cudaEvent_t e0, e1;
   CK(cudaEventCreate(&e0));
@@ -562,7 +561,8 @@ int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
       stage<R>(h, a, st);
     }
   };
-  auto time_one = [&](double* us) -> int {
+  auto time_one = [&](int f, double* us) -> int {
+    h->form = f;
     constexpr int N = 12;
     chain(h->stream, 1);
     if (cudaGetLastError() != cudaSuccess) {  // launch rejected (configuration): form unavailable
@@ -585,21 +585,12 @@ int autotune(cmcg_handle* h, int first, int nforms, int overlap) {
     return CMCG_OK;
   };
   h->pdl = overlap != 2;
-  double best = 1e300;
-  int bestf = first;
-  for (int f = first; f < first + nforms; ++f) {
-    h->form = f;
-    double us;
-    const int rc = time_one(&us);
-    if (rc) return rc;
-    h->tune_us[f] = us;
-    if (us >= 0 && us < best) {
-      best = us;
-      bestf = f;
-    }
-  }
-  h->form = bestf;
-  h->tune_us[7] = h->tune_us[bestf];
+  int form = -1;
+  const int rc = choose_form(h->prec == CMCG_FP32, h->q, h->tune_us, &form, time_one);
+  if (rc) return rc;
+  if (form < 0) return CMCG_ERR_CUDA;  // no form can be launched
+  h->form = form;
+  h->tune_us[7] = h->tune_us[form];
   for (auto it = h->graph_exec.begin(); it != h->graph_exec.end();) {  // the chains' graphs
     if (std::get<0>(it->first) >= TUNE_KIND) {
       cudaGraphExecDestroy(it->second);
@@ -1368,12 +1359,7 @@ int create_impl(int nprob, const cmcg_problem* probs, const cmcg_options* opt_in
     h->form = opt.stage_variant - 1;
     h->pdl = opt.stage_overlap != 2;
   } else {
-    // P3 in FP32 always takes the tensor-core form (16.5 us per stage of 12,288 tetrahedra against 27 for
-    // the best other one, 37 against 95 at 48,000), P1 and P2 one of the others (P2: 22 us against 31
-    // at 81,648 tetrahedra): the arithmetic does not depend on what was measured.
-    if (h->prec == CMCG_FP64) rc = autotune<double>(h, 0, STAGE_FORMS_F64, opt.stage_overlap);
-    else if (h->q == 3) rc = autotune<float>(h, STAGE_FORM_TC, 1, opt.stage_overlap);
-    else rc = autotune<float>(h, 0, STAGE_FORM_TC, opt.stage_overlap);
+    rc = h->prec == CMCG_FP32 ? autotune<float>(h, opt.stage_overlap) : autotune<double>(h, opt.stage_overlap);
     if (rc) return fail(rc);
   }
   h->launches = 0;

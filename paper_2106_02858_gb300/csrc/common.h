@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/cmcg.h"
+#include "stage_forms.h"
 
 namespace cmcg {
 
@@ -174,15 +175,8 @@ struct StageArgs {
 };
 
 // Kernel launchers, one translation unit per order.
-// form: stage-kernel form.  FP32: 0, 1, 2 = one warp per half tile (two threads per
-// tetrahedron) with at least 12, 16, 24 resident warps per SM; 3, 4 = two warps
-// per half tile with at least 12, 16; 5 = four warps per half tile; 6 = tensor-core
-// contractions (tcgen05, 3xTF32).  FP64: 0, 1, 2 = one, two, four warps per half tile.
-// pdl: launch with programmatic stream serialisation (the stage overlaps the
-// previous stage's tail).  nsm: the device's SMs.
-constexpr int STAGE_FORMS_F32 = 7;
-constexpr int STAGE_FORM_TC = 6;
-constexpr int STAGE_FORMS_F64 = 3;
+// form: stage-kernel form (stage_forms.h).  pdl: launch with programmatic stream serialisation (the
+// stage overlaps the previous stage's tail).  nsm: the device's SMs.
 template <int Q, typename R>
 void launch_stage(const StageArgs<R>& a, cudaStream_t s, int form, bool pdl, int nsm);
 template <int Q>
