@@ -84,6 +84,9 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// Every sum of products here, in dg_stage_nodal.cuh and in dg_stage_bern.cuh is written as fma: what the
+// compiler would fuse by itself may differ between the forms, which have to give the same bits.
+//
 // The conductivity, source and impedance-face terms of Phi on the output values n0 .. n0 + NN - 1
 // of the thread (own: its place in the field layout, the partner's is own ^ 1).  The source on the
 // E rows is, at the stage time, Re(J e^{i w t}) = s_cos J_re - s_sin J_im, or, in a sweep driven at
@@ -100,7 +103,7 @@ __device__ __forceinline__ void add_source(R (&phi)[NN], const R (&jv)[NN], R cs
 #pragma unroll
   for (int n = 0; n < NN; ++n) {
     const R re = __shfl_xor_sync(0xffffffffu, jv[n], 1);
-    if (half) phi[n] += cs * re - sn * jv[n];
+    if (half) phi[n] += fma(cs, re, -(sn * jv[n]));
   }
 }
 // Component c.
@@ -110,7 +113,7 @@ __device__ __forceinline__ void add_data(R (&phi)[NN], const R (&jv)[NN], const 
   const int64_t off = (own ^ 1) + (c * NPQ + n0) * 32;
   if (a.sigma && half) {  // Phi_E -= (sigma / eps) E (E is not flipped by Sigma)
 #pragma unroll
-    for (int n = 0; n < NN; ++n) phi[n] -= sigma * a.vin[off + n * 32];
+    for (int n = 0; n < NN; ++n) phi[n] = fma(-sigma, a.vin[off + n * 32], phi[n]);
   }
   if (a.j) {
     if (a.nharm <= 0) {
@@ -126,7 +129,7 @@ __device__ __forceinline__ void add_data(R (&phi)[NN], const R (&jv)[NN], const 
   }
   if (a.bre) {  // impedance-face data, lifted (source sweeps only)
 #pragma unroll
-    for (int n = 0; n < NN; ++n) phi[n] += cf.s_cos * a.bre[off + n * 32] - cf.s_sin * a.bim[off + n * 32];
+    for (int n = 0; n < NN; ++n) phi[n] += fma(cf.s_cos, a.bre[off + n * 32], -(cf.s_sin * a.bim[off + n * 32]));
   }
 }
 
@@ -151,8 +154,8 @@ __device__ __forceinline__ void accumulate_filter(const StageArgs<R>& a, const S
 #pragma unroll
     for (int n = 0; n < 10; ++n)
       if (n0 + n < NN) {
-        a.fre[off + (n0 + n) * 32] = fr[n] + (cf.fa_re * u[n] + cf.fb_re * phi[n0 + n]);
-        a.fim[off + (n0 + n) * 32] = fi[n] + (cf.fa_im * u[n] + cf.fb_im * phi[n0 + n]);
+        a.fre[off + (n0 + n) * 32] = fr[n] + fma(cf.fa_re, u[n], cf.fb_re * phi[n0 + n]);
+        a.fim[off + (n0 + n) * 32] = fi[n] + fma(cf.fa_im, u[n], cf.fb_im * phi[n0 + n]);
       }
   }
 }

@@ -284,6 +284,6 @@ __device__ __forceinline__ void bern_part(const StageArgs<double>& a, int64_t ht
   }
   if (a.out) {
 #pragma unroll
-    for (int k = 0; k < NO; ++k) a.out[(own ^ 1) + (O0 + k) * 32] = bv[k] + cf.c_out * out[k];
+    for (int k = 0; k < NO; ++k) a.out[(own ^ 1) + (O0 + k) * 32] = fma(cf.c_out, out[k], bv[k]);
   }
 }

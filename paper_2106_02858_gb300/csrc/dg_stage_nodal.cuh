@@ -215,7 +215,7 @@ __device__ __forceinline__ void nodal_part(const StageArgs<float>& a, int64_t ht
         }
       }
       // d/dx_ax of component c = sum_b G[b][ax] d[b][c]
-      auto dx = [&](int ax, int c) { return G[0 * 3 + ax] * d[0][c] + G[1 * 3 + ax] * d[1][c] + G[2 * 3 + ax] * d[2][c]; };
+      auto dx = [&](int ax, int c) { return fmaf(G[2 * 3 + ax], d[2][c], fmaf(G[0 * 3 + ax], d[0][c], G[1 * 3 + ax] * d[1][c])); };
       phi[0][ii] = sv * (dx(1, 2) - dx(2, 1));
       phi[1][ii] = sv * (dx(2, 0) - dx(0, 2));
       phi[2][ii] = sv * (dx(0, 1) - dx(1, 0));
@@ -309,7 +309,7 @@ __device__ __forceinline__ void nodal_part(const StageArgs<float>& a, int64_t ht
     if (a.fre) accumulate_filter<float, NN>(a, cf, phi[c], own, c, I0);  // forward sweeps with the filter only
     if (a.out) {
 #pragma unroll
-      for (int n = 0; n < NN; ++n) a.out[(own ^ 1) + (c * NP + I0 + n) * 32] = bv[c][n] + cf.c_out * phi[c][n];
+      for (int n = 0; n < NN; ++n) a.out[(own ^ 1) + (c * NP + I0 + n) * 32] = fmaf(cf.c_out, phi[c][n], bv[c][n]);
     }
   }
 }
