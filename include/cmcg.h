@@ -342,7 +342,7 @@ int cmcg_solve_multifreq(cmcg_handle* h, int nharm, const int* harmonics, const 
  * double[nt][6][Np] host arrays. */
 int cmcg_inner(cmcg_handle* h, const double* u, const double* v, double* out);
 
-/* Largest nt accepted by cmcg_inner_noalloc. */
+/* Largest nt accepted by cmcg_inner_noalloc (a limit of the interface: its scratch does not grow with nt). */
 #define CMCG_NOALLOC_MAX_TETS 1048576
 
 /* The paper has no counterpart: this is cmcg_inner without a handle and
@@ -358,7 +358,7 @@ int cmcg_inner(cmcg_handle* h, const double* u, const double* v, double* out);
  *   (six times the volume of K);  out: device double[1].
  * Runs on `stream` (a cudaStream_t, NULL = legacy default stream) of the
  * current device and returns once its two kernels are launched; *out is valid
- * when the stream reaches that point.  It reduces through a 64 KiB static
+ * when the stream reaches that point.  It reduces through a 19 KiB static
  * device array that every GPU loading the library holds until the process
  * exits.  The first call on a device does a one-time set-up (looks up the
  * array's device address); make that first call before any stream capture.

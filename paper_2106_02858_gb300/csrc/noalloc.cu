@@ -10,7 +10,7 @@
 // through a per-handle block-partials buffer allocated by cmcg_create; this
 // variant reduces through one file-scope array instead.
 //
-// The array (NA_MAX_BLOCKS doubles, 64 KiB) is static device memory: every
+// The array (NA_BLOCKS doubles, 19 KiB) is static device memory: every
 // GPU that loads the library holds it until the process exits.  Host code only
 // ever sees a stand-in for its name, so the device address is fetched with
 // cudaGetSymbolAddress once per device, with that device current, and passed
@@ -26,20 +26,18 @@ namespace cmcg {
 namespace {
 
 constexpr int NA_THREADS = 128;        // one partial per block
-constexpr int NA_MAX_BLOCKS = 8192;    // 8192 doubles = 64 KiB of static scratch
-// At most; larger meshes give every thread of every block the same number of components more: with
+// Blocks, at most; larger meshes give every thread of every block the same number of components more: with
 // the grid's stride, and the last pass partly idle, the figure below is 79 us instead of 68.
 constexpr int NA_BLOCKS = 152 * 16;
-static_assert(NA_BLOCKS <= NA_MAX_BLOCKS, "scratch");
-static_assert(int64_t(128) * NA_MAX_BLOCKS == CMCG_NOALLOC_MAX_TETS, "limit mismatch");
 
-static __device__ __align__(256) double g_na_partials[NA_MAX_BLOCKS];
+static __device__ __align__(256) double g_na_partials[NA_BLOCKS];
 
 // x^T M y of one component's nodal values on the unit tetrahedron.  M commutes with the renumberings
 // of the four vertices, so it is a short form in sums that belong to a vertex i: s_i (P2: the midpoints
 // of its three edges), a_i, b_i (P3: the near and the far nodes of its three edges), f_i (P3: the node
 // of the opposite face), their totals over i, and the plain product over edge nodes, with whole
-// coefficients (exact: they follow from the simplex integrals):
+// coefficients (they follow from the simplex integrals; na_form evaluates P2's first line with 2/5 and
+// 7.2 in their place, rounded):
 //   P1 (x 120):    sum_i v v' + V V'
 //   P2 (x 2520):   sum_i (5 v v' + 2 (v s' + s v') + 8 s s') + V V' - 3 (V S' + S V') + 2 S S' + 8 sum_e e e'
 //   P3 (x 26880):  sum_i (14 v v' - 15 (v a' + a v') + 3 (v b' + b v') + 18 (v f' + f v') + 54 a a'
@@ -207,7 +205,7 @@ extern "C" int cmcg_inner_noalloc(int order, int64_t nt, const double* u, const 
                                   double* out, void* stream) {
   using namespace cmcg;
   if (order < 1 || order > 3 || nt < 1 || !u || !v || !w || !out) return CMCG_ERR_INVALID_ARG;
-  if (nt > CMCG_NOALLOC_MAX_TETS) return CMCG_ERR_INVALID_ARG;  // beyond the static scratch
+  if (nt > CMCG_NOALLOC_MAX_TETS) return CMCG_ERR_INVALID_ARG;  // the interface's limit
   int device = 0;
   if (cudaGetDevice(&device) != cudaSuccess) return CMCG_ERR_NO_DEVICE;
   if (device < 0 || device >= 64) return CMCG_ERR_INVALID_ARG;
