@@ -369,9 +369,9 @@ void stage(cmcg_handle* h, StageArgs<R>& a, cudaStream_t st) {
   a.tprob = h->tprob;
   a.flip = h->alternate ? h->flip ^= 1 : 0;
   a.nsm = h->nsm;
-  if (h->q == 1) launch_stage<1, R>(a, st, h->form, h->pdl, h->nsm);
-  else if (h->q == 2) launch_stage<2, R>(a, st, h->form, h->pdl, h->nsm);
-  else launch_stage<3, R>(a, st, h->form, h->pdl, h->nsm);
+  if (h->q == 1) launch_stage<1, R>(a, st, h->form, h->pdl);
+  else if (h->q == 2) launch_stage<2, R>(a, st, h->form, h->pdl);
+  else launch_stage<3, R>(a, st, h->form, h->pdl);
 }
 template <typename R>
 void stage(cmcg_handle* h, StageArgs<R>& a) {

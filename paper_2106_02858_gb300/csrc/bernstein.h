@@ -1,5 +1,5 @@
-// The Bernstein form of the degree-q polynomials on a tetrahedron, the basis of every field
-// vector inside a handle: coefficient c_b of B_b = q! / (b0! b1! b2! b3!) l0^b0 l1^b1 l2^b2 l3^b3
+// The Bernstein form of the degree-q polynomials on a tetrahedron, the basis of the field vectors
+// inside an FP64 handle (FP32 handles hold nodal values): coefficient c_b of B_b = q! / (b0! b1! b2! b3!) l0^b0 l1^b1 l2^b2 l3^b3
 // sits at the place of the equispaced node b / q (lattice_index order), so faces, permutations
 // and neighbour codes are those of the nodes.  In this basis the operators of the DG scheme are
 // sparse (for the nodal values they are dense):

@@ -176,9 +176,9 @@ struct StageArgs {
 
 // Kernel launchers, one translation unit per order.
 // form: stage-kernel form (stage_forms.h).  pdl: launch with programmatic stream serialisation (the
-// stage overlaps the previous stage's tail).  nsm: the device's SMs.
+// stage overlaps the previous stage's tail).
 template <int Q, typename R>
-void launch_stage(const StageArgs<R>& a, cudaStream_t s, int form, bool pdl, int nsm);
+void launch_stage(const StageArgs<R>& a, cudaStream_t s, int form, bool pdl);
 template <int Q>
 void upload_constants(const RefMats& rm);
 

@@ -239,9 +239,12 @@ constexpr size_t stage_smem() {
 // Shared memory per block such that no SM takes more blocks than an even spread over the SMs gives it,
 // for grids of more blocks than SMs (P1 FP32 24,576 tetrahedra 1,190 us a sweep without it, 1,040 so; 48,000
 // 2,121 and 1,889).  Smaller grids are left alone: a whole SM to a block keeps other handles' kernels
-// out (four handles of 4,374 P1 tetrahedra on four streams 1.29 ms so, 0.83 without).  P2 FP32 with two or
-// four warps a half tile loses by it (1,296 tetrahedra: 994 and 1,160 us).
-constexpr size_t SM_SHARED = 228 * 1024, BLOCK_RESERVED = 1024, MAX_DYNAMIC = 128 * 1024;
+// out (four handles of 4,374 P1 tetrahedra on four streams 1.29 ms so, 0.83 without).  P2 and P3 FP32 with two or
+// four warps a half tile gain or lose by it (us a sweep without and with, P2 3,072 tetrahedra and four
+// warps 1,838 and 1,991, 7,986 and two warps 2,468 and 2,334); the one-warp forms are faster at all these
+// sizes (1,311 and 1,890), so they are left alone.  The P3 tensor-core stage takes more than any pad.
+constexpr size_t SM_SHARED = 228 * 1024, BLOCK_RESERVED = 1024;
+constexpr size_t MAX_DYNAMIC = 96 * 1024;  // above the largest need (P3 tensor cores 94 KB, FP64 73 KB) and pad (77 KB)
 inline size_t spread_smem(size_t need, int64_t blocks, int nsm) {
   const int64_t per_sm = (blocks + nsm - 1) / nsm;
   const size_t pad = SM_SHARED / size_t(per_sm + 1) / 128 * 128 + 128 - BLOCK_RESERVED;  // per_sm + 1 such blocks don't fit
@@ -264,12 +267,13 @@ void launch_k(void (*k)(Arg), unsigned blocks, unsigned threads, size_t smem, cu
 }
 
 template <typename R, int SPLIT, int WARPS, int MINB>
-void launch_form(const StageArgs<R>& a, cudaStream_t s, bool pdl, int nsm) {
+void launch_form(const StageArgs<R>& a, cudaStream_t s, bool pdl) {
   constexpr bool spread = sizeof(R) == 8 || SPLIT == 1 || CMCG_Q == 1;
   constexpr size_t need = stage_smem<R, SPLIT, WARPS>();
+  static_assert(need <= MAX_DYNAMIC, "shared memory");
   const int64_t warps = a.nti / HTILE * SPLIT, blocks = (warps + WARPS - 1) / WARPS;
   launch_k(dg_stage_kernel<R, SPLIT, WARPS, MINB>, unsigned(blocks), 32 * WARPS,
-           spread ? spread_smem(need, blocks, nsm) : need, s, pdl, a);
+           spread ? spread_smem(need, blocks, a.nsm) : need, s, pdl, a);
 }
 template <typename R, int SPLIT, int WARPS, int MINB>
 void allow_smem() {
@@ -280,26 +284,26 @@ void allow_smem() {
 }  // namespace
 
 template <>
-void launch_stage<CMCG_Q, float>(const StageArgs<float>& a, cudaStream_t s, int form, bool pdl, int nsm) {
+void launch_stage<CMCG_Q, float>(const StageArgs<float>& a, cudaStream_t s, int form, bool pdl) {
   switch (form) {
-    case 1: launch_form<float, 1, 4, 4>(a, s, pdl, nsm); break;
-    case 2: launch_form<float, 1, 4, 6>(a, s, pdl, nsm); break;
-    case 3: launch_form<float, 2, 4, 3>(a, s, pdl, nsm); break;
-    case 4: launch_form<float, 2, 4, 4>(a, s, pdl, nsm); break;
-    case 5: launch_form<float, 4, 4, 4>(a, s, pdl, nsm); break;
+    case 1: launch_form<float, 1, 4, 4>(a, s, pdl); break;
+    case 2: launch_form<float, 1, 4, 6>(a, s, pdl); break;
+    case 3: launch_form<float, 2, 4, 3>(a, s, pdl); break;
+    case 4: launch_form<float, 2, 4, 4>(a, s, pdl); break;
+    case 5: launch_form<float, 4, 4, 4>(a, s, pdl); break;
     case STAGE_FORM_TC:
       launch_k(dg_stage_tc<TC_MINB>, unsigned((a.nti + TC_TETS - 1) / TC_TETS), TC_THREADS,
-               spread_smem(tc_smem(), (a.nti + TC_TETS - 1) / TC_TETS, nsm), s, pdl, a);
+               spread_smem(tc_smem(), (a.nti + TC_TETS - 1) / TC_TETS, a.nsm), s, pdl, a);
       break;
-    default: launch_form<float, 1, 2, 6>(a, s, pdl, nsm); break;
+    default: launch_form<float, 1, 2, 6>(a, s, pdl); break;
   }
 }
 template <>
-void launch_stage<CMCG_Q, double>(const StageArgs<double>& a, cudaStream_t s, int form, bool pdl, int nsm) {
+void launch_stage<CMCG_Q, double>(const StageArgs<double>& a, cudaStream_t s, int form, bool pdl) {
   switch (form) {
-    case 1: launch_form<double, 2, 2, 1>(a, s, pdl, nsm); break;
-    case 2: launch_form<double, 4, 4, 1>(a, s, pdl, nsm); break;
-    default: launch_form<double, 1, 4, 1>(a, s, pdl, nsm); break;
+    case 1: launch_form<double, 2, 2, 1>(a, s, pdl); break;
+    case 2: launch_form<double, 4, 4, 1>(a, s, pdl); break;
+    default: launch_form<double, 1, 4, 1>(a, s, pdl); break;
   }
 }
 
@@ -318,6 +322,7 @@ void upload_constants<CMCG_Q>(const RefMats& rm) {
   cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(MAX_DYNAMIC));
   cudaFuncSetAttribute(dg_stage_tc<TC_MINB>, cudaFuncAttributePreferredSharedMemoryCarveout,
                        int(cudaSharedmemCarveoutMaxShared));  // two P3 CTAs per SM need 2 x 95 KB
+  static_assert(tc_smem() <= MAX_DYNAMIC, "shared memory");
   tc_upload_reference(rm);
   std::vector<float> Df, Lf(rm.LIFT.size());  // LIFT: [node][face node]
   for (size_t k = 0; k < Lf.size(); ++k) Lf[(k % (4 * NFPQ)) * NPQ + k / (4 * NFPQ)] = float(rm.LIFT[k]);
