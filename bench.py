@@ -43,6 +43,9 @@ WORKLOAD = ("scatterer 24^3 Kuhn cube minus centred PEC cube (81,648 tets), P2 /
 CG_ITERS_FOR_REFERENCE = 35
 PROFILE_SUMMARY = os.path.join(ROOT, "profiles", "dg_stage_scatterer24_P2_fp32.md")
 STAGE_SRC = os.path.join(ROOT, "paper_2106_02858_gb300", "csrc", "dg_stage.cuh")
+# What else decides the FP32 stage's traffic: its body, the field layout and the arguments, the order of the mesh.
+STAGE_PARTS = [os.path.join(ROOT, "paper_2106_02858_gb300", "csrc", f)
+               for f in ("dg_stage_nodal.cuh", "bernstein.h", "common.h", "setup.cpp")]
 # FP32 stage-kernel forms, indexed by cmcg_options.stage_variant - 1.
 STAGE_FORMS = ["dg_stage_kernel<float, 1, 2, 6>", "dg_stage_kernel<float, 1, 4, 4>", "dg_stage_kernel<float, 1, 4, 6>",
                "dg_stage_kernel<float, 2, 4, 3>", "dg_stage_kernel<float, 2, 4, 4>", "dg_stage_kernel<float, 4, 4, 4>",
@@ -202,7 +205,8 @@ FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 
 def recorded_traffic(stage_variant: int):
     """Per-launch DRAM bytes of the stage kernel from the committed ncu summary, if that
-    summary was taken of the same kernel form with the kernel source unchanged since; else None."""
+    summary was taken of the same kernel form with the kernel source unchanged since; else None.
+    A summary may give the hash of STAGE_PARTS, read one after another, beside that of STAGE_SRC: both must hold then."""
     if not os.path.exists(PROFILE_SUMMARY):
         return None
     txt = open(PROFILE_SUMMARY).read()
@@ -211,8 +215,12 @@ def recorded_traffic(stage_variant: int):
     m_tr = re.search(r"dram bytes per launch \(read \+ write\):\s*([0-9.eE+]+)", txt)
     if not (m_sha and m_tr and m_var) or int(m_var.group(1)) != stage_variant:
         return None
-    sha = hashlib.sha256(open(STAGE_SRC, "rb").read()).hexdigest()
-    return float(m_tr.group(1)) if sha == m_sha.group(1) else None
+    if hashlib.sha256(open(STAGE_SRC, "rb").read()).hexdigest() != m_sha.group(1):
+        return None
+    m_parts = re.search(r"included sources sha256[^:]*:\s*([0-9a-f]{64})", txt)
+    if m_parts and hashlib.sha256(b"".join(open(f, "rb").read() for f in STAGE_PARTS)).hexdigest() != m_parts.group(1):
+        return None
+    return float(m_tr.group(1))
 
 
 # ---------------------------------------------------------------------------------------------
