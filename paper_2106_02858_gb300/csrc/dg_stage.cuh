@@ -113,7 +113,7 @@ __device__ __forceinline__ void add_data(R (&phi)[NN], const R (&jv)[NN], const 
   const int64_t off = (own ^ 1) + (c * NPQ + n0) * 32;
   if (a.sigma && half) {  // Phi_E -= (sigma / eps) E (E is not flipped by Sigma)
 #pragma unroll
-    for (int n = 0; n < NN; ++n) phi[n] = fma(-sigma, a.vin[off + n * 32], phi[n]);
+    for (int n = 0; n < NN; ++n) phi[n] = fma(sigma, -a.vin[off + n * 32], phi[n]);
   }
   if (a.j) {
     if (a.nharm <= 0) {
